@@ -107,25 +107,13 @@ k_build_lo(DevParams P, ClusterDev C, int count, int32_t* __restrict__ ovf, int*
     build_table<E>(P, C, w, sm[warp]);
 }
 
-// A grid of at most OVF_BLOCKS CTAs whose warps take the listed workers in
-// turn: usually the list is empty, and a small grid costs less to launch.
-constexpr int OVF_BLOCKS = 256;
+// Workers beyond 128 requests: a CTA of NW cooperating warps each (a single
+// warp building 512 elements, 16 a lane, took 64 us where 8 warps take 10; 32 a
+// lane do not fit its registers). The workers are `list[0..count)` with count
+// read on the device (count_dev) or given; the grid's CTAs take them in turn
+// (usually there are none, and a small grid costs less to launch).
+constexpr int OVF_BLOCKS = 304;
 
-template <int E>
-__global__ void __launch_bounds__(BUILD_WARPS * 32)
-k_build_ovf(DevParams P, ClusterDev C, const int32_t* __restrict__ ovf, const int* __restrict__ novf)
-{
-    extern __shared__ __align__(16) unsigned char smraw[];
-    BuildSmem<E>* sm = reinterpret_cast<BuildSmem<E>*>(smraw);
-    const int warp = threadIdx.x >> 5;
-    const int n = *novf;
-    for (int idx = blockIdx.x * BUILD_WARPS + warp; idx < n; idx += gridDim.x * BUILD_WARPS)
-        build_table<E>(P, C, ovf[idx], sm[warp]);
-}
-
-// Tables of 1,024 slots: one CTA of NW cooperating warps per worker (a
-// single warp cannot hold 32 elements per lane in registers). The workers are
-// `list[0..count)` with count read on the device (count_dev) or given.
 template <int EW, int NW>
 __global__ void __launch_bounds__(NW * 32)
 k_build_coop(DevParams P, ClusterDev C, const int32_t* __restrict__ list, int count,
@@ -134,9 +122,11 @@ k_build_coop(DevParams P, ClusterDev C, const int32_t* __restrict__ list, int co
     extern __shared__ __align__(16) unsigned char smraw[];
     BuildSmem<EW, NW>& sm = *reinterpret_cast<BuildSmem<EW, NW>*>(smraw);
     const int n = count_dev ? *count_dev : count;
-    if ((int)blockIdx.x >= n) return;  // CTA-uniform
-    const int w = list ? list[blockIdx.x] : (int)blockIdx.x;
-    build_table_fit<EW, NW>(P, C, w, C.n[w], reinterpret_cast<unsigned char*>(&sm));
+    for (int k = blockIdx.x; k < n; k += gridDim.x) {
+        const int w = list ? list[k] : k;
+        build_table_fit<EW, NW>(P, C, w, C.n[w], reinterpret_cast<unsigned char*>(&sm));
+        __syncthreads();  // the scratch is free
+    }
 }
 
 template <auto Kern>
@@ -154,33 +144,22 @@ static cudaError_t build_e(const DevParams& P, const ClusterDev& C, const int32_
     if (count <= 0) return cudaSuccess;
     const int blocks = (count + BUILD_WARPS - 1) / BUILD_WARPS;
     cudaError_t e;
-    if constexpr (E > 16) {
+    if constexpr (E > E_LO) {
         constexpr int EW = E / COOP_NW;
         const size_t sc = sizeof(BuildSmem<EW, COOP_NW>);
         if ((e = allow_smem<k_build_coop<EW, COOP_NW>>(sc)) != cudaSuccess) return e;
+        const int grid = count < OVF_BLOCKS ? count : OVF_BLOCKS;
         if (list) {
-            k_build_coop<EW, COOP_NW><<<count, COOP_NW * 32, sc, st>>>(P, C, list, count, nullptr);
+            k_build_coop<EW, COOP_NW><<<grid, COOP_NW * 32, sc, st>>>(P, C, list, count, nullptr);
             return cudaGetLastError();
         }
         const size_t slo = sizeof(BuildSmem<E_LO>) * BUILD_WARPS;
         if ((e = allow_smem<k_build_lo<E_LO>>(slo)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(C.novf, 0, sizeof(int), st)) != cudaSuccess) return e;
         k_build_lo<E_LO><<<blocks, BUILD_WARPS * 32, slo, st>>>(P, C, count, C.ovf, C.novf, S);
-        k_build_coop<EW, COOP_NW><<<count, COOP_NW * 32, sc, st>>>(P, C, C.ovf, 0, C.novf);
+        k_build_coop<EW, COOP_NW><<<grid, COOP_NW * 32, sc, st>>>(P, C, C.ovf, 0, C.novf);
         return cudaGetLastError();
     } else {
-        if (E > E_LO && !list) {
-            constexpr int EL = E > E_LO ? E_LO : E;
-            const size_t slo = sizeof(BuildSmem<EL>) * BUILD_WARPS;
-            const size_t shi = sizeof(BuildSmem<E>) * BUILD_WARPS;
-            if ((e = allow_smem<k_build_lo<EL>>(slo)) != cudaSuccess) return e;
-            if ((e = allow_smem<k_build_ovf<E>>(shi)) != cudaSuccess) return e;
-            if ((e = cudaMemsetAsync(C.novf, 0, sizeof(int), st)) != cudaSuccess) return e;
-            k_build_lo<EL><<<blocks, BUILD_WARPS * 32, slo, st>>>(P, C, count, C.ovf, C.novf, S);
-            k_build_ovf<E><<<blocks < OVF_BLOCKS ? blocks : OVF_BLOCKS, BUILD_WARPS * 32, shi, st>>>(
-                P, C, C.ovf, C.novf);
-            return cudaGetLastError();
-        }
         const size_t smem = sizeof(BuildSmem<E>) * BUILD_WARPS;
         if ((e = allow_smem<k_build<E>>(smem)) != cudaSuccess) return e;
         k_build<E><<<blocks, BUILD_WARPS * 32, smem, st>>>(P, C, list, count, S);
