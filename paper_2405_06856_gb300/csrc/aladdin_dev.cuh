@@ -529,6 +529,115 @@ __device__ __forceinline__ void add_carry_suffix(Set& st, typename Set::value_ty
     }
 }
 
+// The terms of a table that the placement chain also forms request by request
+// (round_chain.cu): both call these, so that both round alike.
+
+// Cumulative decode time T(x) of iterations 1..x: Sb requests summed over the
+// iterations, SK context tokens (the product with s rounded by itself).
+__device__ __forceinline__ float decode_time(const DevParams& P, float s, float x, float Sb,
+                                             float SK)
+{
+    return __fmul_rn(s, P.c3 * x + P.c2 * Sb + P.k2 * SK);
+}
+
+// Slack sigma_j of a request of r remaining iterations that end at T; base =
+// theta T_dec r + bank.
+__device__ __forceinline__ float slack_base(const DevParams& P, float r, float bank)
+{
+    return fmaf(P.theta_Tdec, r, bank);
+}
+
+// A request finishing with or before the candidate bounds the prompt by a
+// quotient: its slack less the candidate's share of its r iterations (u_j =
+// sigma_j - s * shared_time), and the stall too for one decoding at round
+// start (stallk = k1 P + c1), over the prompt's cost.
+__device__ __forceinline__ float shared_time(const DevParams& P, float r)
+{
+    return P.c2 * r + P.k2 * (0.5f * r * (r + 1.0f));
+}
+__device__ __forceinline__ float shared_slack(float s, float sigma, float shared)
+{
+    return fmaf(-s, shared, sigma);
+}
+__device__ __forceinline__ float stalled_slack(float s, float u, float stallk)
+{
+    return fmaf(-s, stallk, u);
+}
+__device__ __forceinline__ float prompt_cost_new(const DevParams& P, float s, float r)
+{
+    return s * P.k2 * r;
+}
+__device__ __forceinline__ float prompt_cost_ongoing(const DevParams& P, float s, float r)
+{
+    return s * (P.k2 * r + P.k1);
+}
+
+// Row fields of the requests finishing after the candidate and of its own
+// decode bound.
+__device__ __forceinline__ float row_gt(float smS, float inv_s, float stallk)
+{
+    return smS * inv_s - stallk;
+}
+__device__ __forceinline__ float row_b0n(const DevParams& P, float PR, float PRA)
+{
+    return -(P.c2_over_k2 * PR + PRA);
+}
+__device__ __forceinline__ float row_b1(const DevParams& P, float inv_s, float nf, float A)
+{
+    return P.c3_over_k2 + P.c2_over_k2 * nf + A + 0.5f * nf - P.thTdec_over_k2 * inv_s;
+}
+
+// Worker record without its rank: TTFT bounds (the candidate's Zc is +inf on
+// a decode instance, and so is its bound Zc / s - y).
+__device__ __forceinline__ float4 worker_record(const DevParams& P, float inv_s, float off,
+                                                float sumP, float wpmax, int npend)
+{
+    float4 wr;
+    wr.x = inv_s;
+    wr.y = P.decode ? 0.0f : off * inv_s * P.inv_k1 + P.c1_over_k1 + sumP;
+    wr.z = (npend > 0 && !P.decode)
+               ? (P.T_pre - wpmax - off) * inv_s * P.inv_k1 - P.c1_over_k1 - sumP
+               : f_inf();
+    wr.w = 0.0f;
+    return wr;
+}
+
+// Approximate mode: prompt bounds of (d) (stall within the smallest
+// theta-scaled saved decode time dmin) and of (b) (weighted context within
+// theta * l_d(n + 1), Eq. input limit), in fp64, rounded once.
+__device__ __forceinline__ float2 approx_bounds(const DevParams& P, double s_d, double dmin, int n,
+                                                long long sumP, long long sumIn, long long sumPred)
+{
+    float2 wa;
+    if (P.decode) {
+        wa.x = f_inf();  // no prefill, no stall: (d) is vacuous
+    } else {
+        const double tau0 = s_d * (P.k1d * (double)sumP + P.c1d);
+        wa.x = (float)((dmin - tau0) / (s_d * P.k1d));
+    }
+    const double ld = (P.T_decd / s_d - P.c3d - P.c2d * (double)(n + 1)) / P.k2d;
+    wa.y = (float)(P.thetad * ld - ((double)sumIn + P.gammad * (double)sumPred));
+    return wa;
+}
+
+// capacity_norm key: capacity_norm^2 is exact (integer and half-integer terms
+// below 2^53) and non-negative doubles order like their bit patterns; with
+// gamma = 1/2 the same order comes from integers, 4 capacity_norm^2 = (2B)^2 +
+// (2 sum in + sum pred)^2. Code 0 is kept for an unusable worker.
+__device__ __forceinline__ unsigned long long norm_key(const DevParams& P, int n, long long sumIn,
+                                                       long long sumPred)
+{
+    if (P.gammad == 0.5) {
+        const unsigned long long b2 = 2ull * (unsigned long long)n;
+        const unsigned long long s2 = 2ull * (unsigned long long)sumIn + (unsigned long long)sumPred;
+        return b2 * b2 + s2 * s2 + 1ull;
+    }
+    const double kB = (double)n;
+    const double kL = __dadd_rn((double)sumIn, __dmul_rn(P.gammad, (double)sumPred));
+    const double kQ = __dadd_rn(__dmul_rn(kB, kB), __dmul_rn(kL, kL));
+    return (unsigned long long)__double_as_longlong(kQ) + 1ull;
+}
+
 // One table row in its stored form (see the layout above) and its exact
 // integer aggregates.
 struct RowVals {
@@ -552,11 +661,11 @@ __device__ __forceinline__ RowVals make_row(const DevParams& P, float inv_s, int
     o.v0.x = __int_as_float(rho_next);
     o.v0.y = kvB1;
     o.v0.z = kvE;
-    o.v0.w = -(P.c2_over_k2 * (float)PR + (float)PRA);
-    o.v1.x = P.c3_over_k2 + P.c2_over_k2 * nf + (float)A + 0.5f * nf - P.thTdec_over_k2 * inv_s;
+    o.v0.w = row_b0n(P, (float)PR, (float)PRA);
+    o.v1.x = row_b1(P, inv_s, nf, (float)A);
     o.v1.y = -0.5f * nf;
     o.v1.z = pmA;
-    o.v1.w = smS * inv_s - (P.k1 * (float)P_pend + P.c1);
+    o.v1.w = row_gt(smS, inv_s, P.k1 * (float)P_pend + P.c1);
     o.ext = make_float2(pmAp, smSp * inv_s);
     o.aux.PM = PM;
     o.aux.SM = SM;
@@ -581,8 +690,9 @@ __device__ __forceinline__ void store_row(const ClusterDev& C, long long rowid, 
 // Shared-memory copies of one worker's breakpoints, record and key, kept by
 // the sliced placement round (pointers to this worker's entries).
 struct SliceCache {
-    unsigned short* rho;  // rho_{q+1} - 1 of rows q = 0..min(R, rc)-1
-    int rc;               // rows held
+    unsigned short* rho;  // sample i: rho_{q+1} - 1 of row q = ((i + 1) << shift) - 1 < R
+    int rc;               // samples held
+    int shift;            // every (1 << shift)-th row is sampled
     int* R;
     float4* wrec;
     unsigned long long* key;
@@ -735,9 +845,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
         npend = combine_warps<NW>(sm.pi[0], OpAdd<int>(), 0);
         bad = combine_warps<NW>(sm.pi[1], OpMax<int>(), 0);
     }
-    // Approximate mode: prompt bounds of (d) (stall within the smallest
-    // theta-scaled saved decode time) and of (b) (weighted context within
-    // theta * l_d(n + 1), Eq. input limit), in fp64, rounded once.
+    // Approximate mode: the worker's bounds of (d) and (b).
     float2 wa = make_float2(0.0f, 0.0f);
     if (P.approx) {
         double dmin = __longlong_as_double(0x7ff0000000000000ll);  // +inf: nothing decoding
@@ -757,40 +865,16 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             group_sync<NW, BAR>();
             dmin = combine_warps<NW>(sm.pdm, OpMin<double>(), dmin);
         }
-        const double s_d = C.scaled[w];
-        if (P.decode) {
-            wa.x = f_inf();  // no prefill, no stall: (d) is vacuous
-        } else {
-            const double tau0 = s_d * (P.k1d * (double)sumP + P.c1d);
-            wa.x = (float)((dmin - tau0) / (s_d * P.k1d));
-        }
-        const double ld = (P.T_decd / s_d - P.c3d - P.c2d * (double)(n + 1)) / P.k2d;
-        wa.y = (float)(P.thetad * ld - ((double)sumIn + P.gammad * (double)sumPred));
+        wa = approx_bounds(P, C.scaled[w], dmin, n, sumP, sumIn, sumPred);
     }
 
-    // capacity_norm key (one lane; code 0 is kept for a worker holding an
-    // invalid request): capacity_norm^2 is exact (integer and half-integer
-    // terms below 2^53) and non-negative doubles order like their bit
-    // patterns; with gamma = 1/2 the same order comes from integers.
+    // capacity_norm key (one lane; 0 for a worker holding an invalid request).
     // Row 0, the record and the key are written by the last lane of the last
     // warp, which holds the highest elements (often padding) and so has the
     // fewest rows of its own to write.
     const bool row0_lane = q == NW - 1 && lane == 31;
     unsigned long long kq = 0ull;
-    if (row0_lane && !bad) {
-        if (P.gammad == 0.5) {
-            // 4 capacity_norm^2 = (2B)^2 + (2 sum in + sum pred)^2 in integers
-            // (the same order and ties as the exact double value)
-            const unsigned long long b2 = 2ull * (unsigned long long)n;
-            const unsigned long long s2 = 2ull * (unsigned long long)sumIn + (unsigned long long)sumPred;
-            kq = b2 * b2 + s2 * s2 + 1ull;
-        } else {
-            const double kB = (double)n;
-            const double kL = __dadd_rn((double)sumIn, __dmul_rn(P.gammad, (double)sumPred));
-            const double kQ = __dadd_rn(__dmul_rn(kB, kB), __dmul_rn(kL, kL));
-            kq = (unsigned long long)__double_as_longlong(kQ) + 1ull;
-        }
-    }
+    if (row0_lane && !bad) kq = norm_key(P, n, sumIn, sumPred);
 
     constexpr int N = BuildSmem<EW, NW>::N;
     // Cooperative builds of up to 256 slots rank every key by counting the
@@ -1058,13 +1142,13 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             const long long A = tot_a - pre_a[e];
             const long long Sb = pre_r[e] + rr * np;
             const long long SK = pre_ra[e] + np * (rr * (rr + 1) / 2) + rr * A;
-            sm.Tp[rowid[e]] = s * (P.c3 * (float)rr + P.c2 * (float)Sb + P.k2 * (float)SK);
+            sm.Tp[rowid[e]] = decode_time(P, s, (float)rr, (float)Sb, (float)SK);
         }
     }
     group_sync<NW, BAR>();
 
     // Per-request bounds and slacks.
-    const float stall0 = s * (P.k1 * (float)sumP + P.c1);
+    const float stallk = P.k1 * (float)sumP + P.c1;
     float pmA[E], pmAp[E], smS[E], smSp[E];
     long long PMx[E], SMx[E];
 #pragma unroll
@@ -1080,13 +1164,13 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
         if (valid) {
             const float rf = (float)r[e];
             const float Tj = sm.Tp[rowid[e]];
-            const float sigma = P.theta_Tdec * rf + bank[e] - Tj;
-            const float u = sigma - s * (P.c2 * rf + P.k2 * (0.5f * rf * (rf + 1.0f)));
+            const float sigma = slack_base(P, rf, bank[e]) - Tj;
+            const float u = shared_slack(s, sigma, shared_time(P, rf));
             if (pd[e]) {
-                pmAp[e] = u / (s * P.k2 * rf);
+                pmAp[e] = u / prompt_cost_new(P, s, rf);
                 smSp[e] = sigma;
             } else {
-                pmA[e] = (u - stall0) / (s * (P.k2 * rf + P.k1));
+                pmA[e] = stalled_slack(s, u, stallk) / prompt_cost_ongoing(P, s, rf);
                 smS[e] = sigma;
             }
         }
@@ -1125,15 +1209,8 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     const float smSp0 = s_smSp.total;
     const long long SM0 = s_SM.total;
 
-    // Worker record (every lane; the first lane stores it).
-    float4 wr;
-    wr.x = inv_s;
-    // TTFT bounds (the candidate's Zc is +inf on a decode instance, and so is
-    // its bound Zc / s - wr.y)
-    wr.y = P.decode ? 0.0f : off * inv_s * P.inv_k1 + P.c1_over_k1 + (float)sumP;
-    wr.z = (npend > 0 && !P.decode)
-               ? (P.T_pre - wpmax - off) * inv_s * P.inv_k1 - P.c1_over_k1 - (float)sumP
-               : f_inf();
+    // Worker record (every lane; row 0's lane stores it).
+    float4 wr = worker_record(P, inv_s, off, (float)sumP, wpmax, npend);
     wr.w = rank_bits;
     const bool want = cand != nullptr && cand->valid;
     const int rc = want ? cand->ri : 0;
@@ -1155,8 +1232,11 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
                 const RowVals o = make_row(P, inv_s, M, sumP, r[e], nxt, np, A, pre_r[e], pre_ra[e],
                                            PMx[e], SM, pmA[e], pmAp[e], smS[e], smSp[e]);
                 if constexpr (!EVAL) store_row(C, rowbase + rowid[e], o, P.want_aux != 0);
-                if (cache && rowid[e] < R && rowid[e] < cache->rc)
-                    cache->rho[rowid[e]] = (unsigned short)(nxt - 1);
+                if (cache) {
+                    const int q1 = rowid[e] + 1, sh = cache->shift, i = (q1 >> sh) - 1;
+                    if (rowid[e] < R && i >= 0 && i < cache->rc && (q1 & ((1 << sh) - 1)) == 0)
+                        cache->rho[i] = (unsigned short)(nxt - 1);
+                }
                 if (want && r[e] <= rc && rc < nxt) {
                     float m;
                     cf = eval_pair_mode(P.approx, o.v0, o.v1, o.ext, wr, wa, *cand, m);
@@ -1192,7 +1272,8 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             C.key[w] = kq;
         }
         if (cache) {
-            if (!bad && n > 0 && R > 0) cache->rho[0] = (unsigned short)(r0 - 1);
+            if (!bad && n > 0 && R > 0 && cache->shift == 0)
+                cache->rho[0] = (unsigned short)(r0 - 1);
             *cache->R = bad ? 0 : R;
             *cache->wrec = wr;
             *cache->key = kq;

@@ -117,24 +117,27 @@ cudaError_t launch_round(const DevParams& P, const ClusterDev& C, const RoundIO&
 // holds at 1,024 slots, or a failed device query).
 int round_ctas(int W, int cap, int K, bool single_cta);
 
-// Scratch of the incremental round (grow-only, owned by the cluster).
-struct RoundIncBuffers {
-    uint8_t* flags;        // [chunk][(W + 31) & ~31] rank-order flags of the round-start state
+// Scratch of the placement chain (grow-only, owned by the cluster).
+struct RoundChainBuffers {
+    uint8_t* flags;        // [chunk][(W + 31) & ~31] rank-order flags of the round-start
+                           // state, or nullptr (round_chain_flag_bytes is 0)
     void* rank;            // [W] 16-byte rank entries
     int* c_stop;           // one int
     ScoreBuffers score;    // candidate preparation of the pre-scoring (chunk candidates)
 };
-// Bytes of the incremental round's flag buffer for n_cand candidates (0: the
-// incremental round does not apply and needs nothing).
-size_t round_inc_flag_bytes(const DevParams& P, const ClusterDev& C, const RoundIO& io);
-// K4, incremental (direct-mode best-fit rounds of one scheduling group): every
-// candidate scored against the round-start state, then a single-CTA chain
-// that re-scores only the workers it modified; the sliced round finishes any
-// candidates left when the modified workers outgrow shared memory. *used =
-// false: not applicable (trace mode, several groups, the wait test hook),
-// nothing launched.
-cudaError_t launch_round_inc(const DevParams& P, const ClusterDev& C, const RoundIO& io,
-                             const RoundIncBuffers& B, cudaStream_t st, bool* used);
+// Bytes of the chain's flag buffer for a direct-mode round (0: it evaluates
+// workers as it goes and needs none).
+size_t round_chain_flag_bytes(const DevParams& P, const ClusterDev& C, const RoundIO& io);
+// K4 as a chain (round_chain.cu): direct-mode best-fit rounds, of one
+// scheduling group (the sliced round finishes any candidates left when the
+// modified workers outgrow shared memory) or of several (one CTA each), and
+// trace-mode rounds (B unused). *used = false: not applicable (the wait test
+// hook, or a group or simulation of more workers than one CTA holds), nothing
+// launched.
+cudaError_t launch_round_chain(const DevParams& P, const ClusterDev& C, const RoundIO& io,
+                               const RoundChainBuffers* B, cudaStream_t st, bool* used);
+// Whether the chain serves trace-mode rounds of W workers of cap slots.
+bool round_chain_serves_sim(int W, int cap, int K);
 
 // Attributes of the current device that launches size themselves by, read
 // once per device and cached (thread-safe).

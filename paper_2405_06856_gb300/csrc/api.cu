@@ -212,7 +212,7 @@ struct aladdin_cluster {
     DevBuf sorted, hist, best;
     DevBuf s_in, s_pred, s_wait, s_flags, s_margin, s_arg, s_kv, s_tc, s_place;
     DevBuf s_off, s_rin, s_rgen, s_rpred, s_rtdec;
-    DevBuf r_flags, r_rank, r_stop;  // incremental placement round
+    DevBuf r_flags, r_rank, r_stop;  // placement chain
     unsigned long long* d_stats = nullptr;
     int* d_status = nullptr;
     void* d_xround = nullptr;  // exchange buffer of the sliced placement round
@@ -280,7 +280,7 @@ struct aladdin_cluster {
         }
         DevBuf* bufs[] = {&sorted, &hist, &best, &s_in, &s_pred, &s_wait, &s_flags, &s_margin,
                           &s_arg, &s_kv, &s_tc, &s_place, &s_off, &s_rin, &s_rgen, &s_rpred,
-                          &s_rtdec};
+                          &s_rtdec, &r_flags, &r_rank, &r_stop};
         for (DevBuf* b : bufs) b->release();
     }
 };
@@ -844,32 +844,33 @@ try {
     io.rid0 = cl->rid_next;
     cl->rid_last = cl->rid_next;
     cl->aux_valid = false;  // the round rebuilds tables without the aggregates
-    if (cl->hp.policy == ALADDIN_POLICY_BESTFIT && cl->dp.groups > 1) {
-        // independent schedulers: one CTA per group, in parallel
-        CK(launch_round_groups(cl->dp, cl->dev, io, cl->st));
-        CK(launch_rank(cl->dev, cl->st));
-    } else if (cl->hp.policy == ALADDIN_POLICY_BESTFIT) {
-        // incremental round where it applies, the sliced round otherwise
+    if (cl->hp.policy == ALADDIN_POLICY_BESTFIT) {
         io.round_open = cl->round_open ? 1 : 0;
-        bool used = false;
-        const size_t fbytes = round_inc_flag_bytes(cl->dp, cl->dev, io);
+        RoundChainBuffers rb;
+        std::memset(&rb, 0, sizeof(rb));
+        CK(cl->r_rank.ensure(16 * (size_t)cl->W));
+        CK(cl->r_stop.ensure(sizeof(int)));
+        rb.rank = cl->r_rank.p;
+        rb.c_stop = cl->r_stop.as<int>();
+        const size_t fbytes = round_chain_flag_bytes(cl->dp, cl->dev, io);
         if (fbytes > 0) {
             const size_t chunk = fbytes / (size_t)((cl->W + 31) & ~31);
             CK(cl->r_flags.ensure(fbytes));
-            CK(cl->r_rank.ensure(16 * (size_t)cl->W));
-            CK(cl->r_stop.ensure(sizeof(int)));
             CK(cl->sorted.ensure(sizeof(float4) * CAND_REC_F4 * chunk));
             CK(cl->hist.ensure(sizeof(int32_t) * ((size_t)cl->hp.K + 2)));
             CK(cl->best.ensure(sizeof(unsigned int) * chunk));
-            RoundIncBuffers rb;
             rb.flags = cl->r_flags.as<uint8_t>();
-            rb.rank = cl->r_rank.p;
-            rb.c_stop = cl->r_stop.as<int>();
             rb.score = ScoreBuffers{cl->sorted.as<float4>(), cl->hist.as<int32_t>(),
                                     cl->best.as<unsigned int>()};
-            CK(launch_round_inc(cl->dp, cl->dev, io, rb, cl->st, &used));
         }
-        if (!used) CK(launch_round(cl->dp, cl->dev, io, cl->st));
+        // the chain where it applies; otherwise one CTA per group or the
+        // sliced round
+        bool used = false;
+        CK(launch_round_chain(cl->dp, cl->dev, io, &rb, cl->st, &used));
+        if (!used) {
+            if (cl->dp.groups > 1) CK(launch_round_groups(cl->dp, cl->dev, io, cl->st));
+            else CK(launch_round(cl->dp, cl->dev, io, cl->st));
+        }
         CK(launch_rank(cl->dev, cl->st));
     } else {
         // JSQ / power of two: no table is read while placing; every worker's
@@ -1363,8 +1364,13 @@ int simulate_impl(const aladdin_params& p, const aladdin_worker_cfg& cfg, int32_
             io.sim_n = rb_n;
         }
         const bool bestfit = p.policy == ALADDIN_POLICY_BESTFIT;
-        if (bestfit) CK(launch_round(cl.dp, cl.dev, io, st));
-        else CK(launch_round_queue(cl.dp, cl.dev, io, st));
+        if (bestfit) {
+            bool used = false;
+            CK(launch_round_chain(cl.dp, cl.dev, io, nullptr, st, &used));
+            if (!used) CK(launch_round(cl.dp, cl.dev, io, st));
+        } else {
+            CK(launch_round_queue(cl.dp, cl.dev, io, st));
+        }
         if (rebal) {
             // Algorithm 2 on the errors recorded since the previous heartbeat,
             // which then restart from zero
@@ -1441,7 +1447,8 @@ void run_probes(const aladdin_params& p, const aladdin_worker_cfg& cfg, const De
     // probes that no single-CTA round serves must hold the cooperative token
     std::vector<char> need(probes.size(), 0);
     for (size_t k = 0; k < probes.size(); ++k)
-        need[k] = bestfit && round_ctas(probes[k].n, p.b_cap, p.K, true) < 0;
+        need[k] = bestfit && !round_chain_serves_sim(probes[k].n, p.b_cap, p.K) &&
+                  round_ctas(probes[k].n, p.b_cap, p.K, true) < 0;
     auto one = [&](size_t k) {
         SimProbe* q = &probes[k];
         cudaStream_t s = nullptr;

@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(R2_THREADS, 1) k_round2(R2Args A)
     // of the CTA takes the same branch (and the same barrier).
     auto rebuild = [&](int w, bool small, const CandRec* cand) -> unsigned {
         const int lw = w - w_lo;
-        SliceCache sc{rho + (long long)lw * rs, rc, &R_s[lw], &wrec_s[lw], &key_s[lw]};
+        SliceCache sc{rho + (long long)lw * rs, rc, 0, &R_s[lw], &wrec_s[lw], &key_s[lw]};
         append(w);
         if constexpr (NW > 4) {
             if (small) {
