@@ -62,7 +62,7 @@ def build(force=False, verbose=False, extra=()):
         return obj
 
     srcs = sources()
-    with concurrent.futures.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with concurrent.futures.ThreadPoolExecutor(max_workers=min(16, len(srcs))) as ex:
         objs = list(ex.map(one, srcs))
     tmp = LIB + ".tmp%d" % os.getpid()
     cmd = [nv, *ARCH, "-shared", "-o", tmp, *objs, "-lcudart", "-lpthread"]

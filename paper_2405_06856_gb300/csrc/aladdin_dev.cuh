@@ -432,7 +432,7 @@ __device__ __forceinline__ T warp_reduce(T v, Op op)
 template <int EW, int NW = 1>
 struct BuildSmem {
     static constexpr int N = 32 * EW * NW;
-    long long kvrho[N + 1];
+    alignas(16) long long kvrho[N + 1];
     int32_t a[N];
     float bank[N];
     float Tp[N + 1];
@@ -443,7 +443,7 @@ struct BuildSmem {
     float pf[7][NW];
     int pi[5][NW];
     unsigned cflag;
-    unsigned newk[8];                 // insertion: the appended keys
+    unsigned newk;                    // insertion: the appended key
     uint8_t pend[N];
 };
 
@@ -702,27 +702,18 @@ struct SliceCache {
 // Called by all lanes of NW warps (warps W0..W0+NW-1 of the CTA when NW > 1,
 // synchronised by named barrier BAR); element x = (q EW + e) 32 + lane of
 // the group's warp q, so 32 EW NW slots are covered. Requests are loaded from
-// the slot arrays, the first n_in of them (the worker's count when n_in < 0);
-// an invalid request (in < 0, gen outside [0, pred), in + pred > K) makes the
-// worker infeasible for every candidate and sets err bit 1. With `cache`, the
-// worker's shared-memory copies are refreshed as well. With a valid `cand`,
-// the candidate is evaluated against the new table by the lane that holds
-// its row, and every lane returns its flags (else 0). EVAL: the evaluation
-// only (a state that is not committed): nothing is written outside `sm`
-// except the state's capacity_norm key into *key_out. INSERT: the last `ins`
-// slots (1 to 3) were appended since the build that left its sorted keys in
-// skey, and are inserted into that order instead of sorting afresh (ins up
-// to INS_MAX). !SKEY:
-// the sorted keys are left in sm.sorted for the caller to store (a caller
-// that runs an evaluation of the same worker beside this build).
-constexpr int INS_MAX = 5;  // appended keys an insertion build takes
-
-template <int EW, int NW = 1, bool INSERT = false, int BAR = 1, int W0 = 0, bool EVAL = false,
-          bool SKEY = true>
+// the slot arrays; an invalid request (in < 0, gen outside [0, pred), in +
+// pred > K) makes the worker infeasible for every candidate and sets err bit 1.
+// With `cache`, the worker's shared-memory copies are refreshed as well. With a
+// valid `cand`, the candidate is evaluated against the new table by the lane
+// that holds its row, and every lane returns its flags (else 0). INSERT: the
+// last request (1) or the last `ins` requests (2) were appended since the
+// build that left its sorted keys in skey, and are inserted into that order
+// instead of sorting afresh.
+template <int EW, int NW = 1, int INSERT = 0, int BAR = 1, int W0 = 0>
 __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
                                 BuildSmem<EW, NW>& sm, const SliceCache* cache = nullptr,
-                                const CandRec* cand = nullptr, int n_in = -1,
-                                unsigned long long* key_out = nullptr, int ins = 1)
+                                const CandRec* cand = nullptr, int ins = 1)
 {
     static_assert(!INSERT || NW > 1, "the insertion path is for cooperative builds");
     constexpr int E = EW;
@@ -735,7 +726,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     // Independent loads first: the slot loads do not wait for n (slots below
     // the capacity lie inside the worker's slot range; those past n are
     // masked). A build may cover more elements than the capacity (padding).
-    const int n = n_in >= 0 ? n_in : C.n[w];
+    const int n = C.n[w];
     const float s = C.scale[w];
     const int M = C.M[w];
     const float off = C.off[w];
@@ -881,68 +872,89 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     // keys below it (keys of valid requests are distinct); larger ones sort
     // each warp's run and merge the runs.
     constexpr bool COUNT_RANK = NW > 1 && N <= 256 && !INSERT;
-    if constexpr (INSERT) {
-        // Insert the appended requests' keys into the previous sorted order
-        // (keys are distinct): a new key lands after the old and new keys
-        // below it, an old key moves up by the new keys below it.
-        const int n0 = n - ins;  // keys of the previous order
+    if constexpr (INSERT == 1) {
+        // Insert the appended request's key into the previous sorted order: it
+        // lands after the keys below it, the others move up by one.
+        const int n0 = n - 1;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = x0 + e * 32 + lane;
             if (x < n0) sm.runs[x] = l_sk[e];
-            if (x >= n0 && x < n) sm.newk[x - n0] = key[e];
+            if (x == n0) sm.newk = key[e];
         }
         group_sync<NW, BAR>();
-        unsigned nk[INS_MAX];
-        int pos[INS_MAX];
-#pragma unroll
-        for (int j = 0; j < INS_MAX; ++j) {
-            nk[j] = j < ins ? sm.newk[j] : 0xffffffffu;
-            pos[j] = 0;
-        }
-#pragma unroll
-        for (int j = 0; j < INS_MAX; ++j) {
-            if (j >= ins) break;  // uniform
-            int lo;  // old keys below nk[j]
-            if constexpr (E == 1) {
-                // one key a thread: a barrier reduction over the group
-                const unsigned below = (x0 + lane < n0 && l_sk[0] < nk[j]) ? 1u : 0u;
-                unsigned cnt;
-                asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n"
-                             " bar.red.popc.u32 %0, %3, %1, p;\n}"
-                             : "=r"(cnt)
-                             : "r"(NW * 32), "r"(below), "n"(BAR)
-                             : "memory");
-                lo = (int)cnt;
-            } else {
-                int hi = n0;
-                lo = 0;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (sm.runs[mid] < nk[j]) lo = mid + 1;
-                    else hi = mid;
-                }
+        const unsigned nk = sm.newk;
+        int lo;  // old keys below nk
+        if constexpr (E == 1) {
+            // one key a thread: a barrier reduction over the group
+            const unsigned below = (x0 + lane < n0 && l_sk[0] < nk) ? 1u : 0u;
+            unsigned cnt;
+            asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n"
+                         " bar.red.popc.u32 %0, %3, %1, p;\n}"
+                         : "=r"(cnt)
+                         : "r"(NW * 32), "r"(below), "n"(BAR)
+                         : "memory");
+            lo = (int)cnt;
+        } else {
+            int hi = n0;
+            lo = 0;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (sm.runs[mid] < nk) lo = mid + 1;
+                else hi = mid;
             }
-            pos[j] = lo;
-#pragma unroll
-            for (int j2 = 0; j2 < INS_MAX; ++j2) pos[j] += (j2 < ins && nk[j2] < nk[j]) ? 1 : 0;
         }
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = x0 + e * 32 + lane;
-            if (x < n0) {
-                const unsigned k = l_sk[e];
-                int sh = 0;
+            if (x < n0) sm.sorted[x + (nk < l_sk[e] ? 1 : 0)] = l_sk[e];
+        }
+        if (q == 0 && lane == 0) sm.sorted[lo] = nk;
+    }
+    if constexpr (INSERT == 2) {
+        // Several appended requests: every key moves up by the appended keys
+        // below it, counted one by one; an appended key also by the old ones,
+        // found by a search.
+        const int n0 = n - ins;
+        unsigned* newk = reinterpret_cast<unsigned*>(sm.kvrho);  // not in use yet
+        const int pad = (ins + 3) & ~3;
 #pragma unroll
-                for (int j = 0; j < INS_MAX; ++j) sh += (j < ins && nk[j] < k) ? 1 : 0;
-                sm.sorted[x + sh] = k;
+        for (int e = 0; e < E; ++e) {
+            const int x = x0 + e * 32 + lane;
+            if (x < n0) sm.runs[x] = l_sk[e];
+            else if (x < n0 + pad) newk[x - n0] = x < n ? key[e] : 0xffffffffu;
+        }
+        for (int j = ins + q * 32 + lane; j < pad; j += 32 * NW) newk[j] = 0xffffffffu;
+        group_sync<NW, BAR>();
+        unsigned mine[E];
+        int at[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int x = x0 + e * 32 + lane;
+            mine[e] = x < n0 ? l_sk[e] : key[e];
+            at[e] = x;
+            if (x >= n0 && x < n) {
+                int lo = 0, hi = n0;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (sm.runs[mid] < mine[e]) lo = mid + 1;
+                    else hi = mid;
+                }
+                at[e] = lo;
             }
         }
-        if (q == 0 && lane < ins) {
+        const uint4* new4 = reinterpret_cast<const uint4*>(newk);
+        for (int k = 0; k < pad / 4; ++k) {
+            const uint4 v = new4[k];
 #pragma unroll
-            for (int j = 0; j < INS_MAX; ++j)
-                if (j == lane) sm.sorted[pos[j]] = nk[j];
+            for (int e = 0; e < E; ++e)
+                at[e] += (v.x < mine[e]) + (v.y < mine[e]) + (v.z < mine[e]) + (v.w < mine[e]);
         }
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (x0 + e * 32 + lane < n) sm.sorted[at[e]] = mine[e];
+    }
+    if constexpr (INSERT != 0) {
         group_sync<NW, BAR>();
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -1062,7 +1074,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int x = x0 + e * 32 + lane;
-        if (!EVAL && SKEY && x < n) C.skey[base + x] = key[e];
+        if (x < n) C.skey[base + x] = key[e];
     }
     // Neighbours in sorted order.
     int rnext[E], first[E], last[E];
@@ -1222,8 +1234,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
         for (int e = 0; e < E; ++e) {
             const int xe = x0 + e * 32 + lane;
             const int nxe = (xe == n - 1) ? 0x7fffffff : rnext[e];
-            // an evaluation build forms only the candidate's row
-            if (last[e] && (!EVAL || (want && r[e] <= rc && rc < nxe))) {
+            if (last[e]) {
                 const int x = xe;
                 const int np = n - (x + 1);
                 const long long A = tot_a - pre_a[e];
@@ -1231,7 +1242,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
                 const long long SM = SMx[e] == LL_NONE ? 0 : SMx[e];
                 const RowVals o = make_row(P, inv_s, M, sumP, r[e], nxt, np, A, pre_r[e], pre_ra[e],
                                            PMx[e], SM, pmA[e], pmAp[e], smS[e], smSp[e]);
-                if constexpr (!EVAL) store_row(C, rowbase + rowid[e], o, P.want_aux != 0);
+                store_row(C, rowbase + rowid[e], o, P.want_aux != 0);
                 if (cache) {
                     const int q1 = rowid[e] + 1, sh = cache->shift, i = (q1 >> sh) - 1;
                     if (rowid[e] < R && i >= 0 && i < cache->rc && (q1 & ((1 << sh) - 1)) == 0)
@@ -1245,32 +1256,28 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             }
         }
     }
-    if (row0_lane && (!EVAL || (want && (bad || n == 0 || rc < r0)))) {
+    if (row0_lane) {
         RowVals o;
         if (!bad) {
             o = make_row(P, inv_s, M, sumP, 0, n > 0 ? r0 : 0x7fffffff, n, tot_a, 0, 0, LL_NONE,
                          SM0 == LL_NONE ? 0 : SM0, f_inf(), f_inf(), smS0, smSp0);
-            if constexpr (!EVAL) C.R[w] = R;
+            C.R[w] = R;
         } else {
             // An invalid request: no candidate fits this worker.
             o = make_row(P, inv_s, M, 0, 0, 0x7fffffff, 0, 0, 0, 0, LL_NONE, (long long)M + 1,
                          f_inf(), f_inf(), f_inf(), f_inf());
-            if constexpr (!EVAL) {
-                C.R[w] = 0;
-                atomicOr(C.err, 1u);
-            }
+            C.R[w] = 0;
+            atomicOr(C.err, 1u);
         }
-        if constexpr (!EVAL) store_row(C, rowbase, o, P.want_aux != 0);
+        store_row(C, rowbase, o, P.want_aux != 0);
         if (want && (bad || n == 0 || rc < r0)) {
             float m;
             cf = eval_pair_mode(P.approx, o.v0, o.v1, o.ext, wr, wa, *cand, m);
             mine = true;
         }
-        if constexpr (!EVAL) {
-            C.wrec[w] = wr;
-            if (P.approx) C.wapx[w] = wa;
-            C.key[w] = kq;
-        }
+        C.wrec[w] = wr;
+        if (P.approx) C.wapx[w] = wa;
+        C.key[w] = kq;
         if (cache) {
             if (!bad && n > 0 && R > 0 && cache->shift == 0)
                 cache->rho[0] = (unsigned short)(r0 - 1);
@@ -1278,9 +1285,6 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             *cache->wrec = wr;
             *cache->key = kq;
         }
-    }
-    if constexpr (EVAL) {
-        if (row0_lane && key_out) *key_out = kq;
     }
     if constexpr (NW > 1) {
         if (mine) sm.cflag = cf;  // exactly one lane of the group holds the row
@@ -1299,31 +1303,24 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
 // elements, not 1,024). smem holds a BuildSmem<EWMAX, NW>; the smaller
 // variants use a prefix of it. n is the worker's current count (uniform over
 // the NW warps).
-template <int EWMAX, int NW, bool INSERT = false, int BAR = 1, int W0 = 0, bool EVAL = false,
-          bool SKEY = true>
+template <int EWMAX, int NW, int INSERT = 0, int BAR = 1, int W0 = 0>
 __device__ __forceinline__ unsigned build_table_fit(const DevParams& P, const ClusterDev& C, int w,
                                                     int n, unsigned char* smem,
                                                     const SliceCache* cache = nullptr,
-                                                    const CandRec* cand = nullptr,
-                                                    unsigned long long* key_out = nullptr,
-                                                    int ins = 1)
+                                                    const CandRec* cand = nullptr, int ins = 1)
 {
-    // an evaluation build is given its count (beyond the worker's own)
-    const int n_in = EVAL ? n : -1;
     if constexpr (EWMAX >= 4) {
         if (n > 64 * NW)  // more than the EW = 2 variant covers
-            return build_table<4, NW, INSERT, BAR, W0, EVAL, SKEY>(
-                P, C, w, *reinterpret_cast<BuildSmem<4, NW>*>(smem), cache, cand, n_in, key_out,
-                ins);
+            return build_table<4, NW, INSERT, BAR, W0>(
+                P, C, w, *reinterpret_cast<BuildSmem<4, NW>*>(smem), cache, cand, ins);
     }
     if constexpr (EWMAX >= 2) {
         if (n > 32 * NW)
-            return build_table<2, NW, INSERT, BAR, W0, EVAL, SKEY>(
-                P, C, w, *reinterpret_cast<BuildSmem<2, NW>*>(smem), cache, cand, n_in, key_out,
-                ins);
+            return build_table<2, NW, INSERT, BAR, W0>(
+                P, C, w, *reinterpret_cast<BuildSmem<2, NW>*>(smem), cache, cand, ins);
     }
-    return build_table<1, NW, INSERT, BAR, W0, EVAL, SKEY>(
-        P, C, w, *reinterpret_cast<BuildSmem<1, NW>*>(smem), cache, cand, n_in, key_out, ins);
+    return build_table<1, NW, INSERT, BAR, W0>(
+        P, C, w, *reinterpret_cast<BuildSmem<1, NW>*>(smem), cache, cand, ins);
 }
 
 }  // namespace aladdin

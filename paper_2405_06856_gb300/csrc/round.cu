@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(R2_THREADS, 1) k_round2(R2Args A)
 {
     constexpr int NW = R2Split<E>::NW, EW = R2Split<E>::EW;
     // the winner's previous sorted order is current: insert its new key
-    constexpr bool NW_INSERT = NW > 1;
+    constexpr int NW_INSERT = NW > 1 ? 1 : 0;
     extern __shared__ __align__(16) unsigned char smraw[];
     R2Smem<E>& sm = *reinterpret_cast<R2Smem<E>*>(smraw);
     const int cap = A.C.cap;
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(R2_THREADS, 1) k_round2(R2Args A)
         if constexpr (NW > 4) {
             if (small) {
                 group_sync<4>();
-                return build_table_fit<1, 4, true>(P, C, w, n_s[lw],
+                return build_table_fit<1, 4, 1>(P, C, w, n_s[lw],
                                                    reinterpret_cast<unsigned char*>(&sm.build),
                                                    &sc, cand);
             }
