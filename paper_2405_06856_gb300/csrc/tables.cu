@@ -129,6 +129,25 @@ k_build_coop(DevParams P, ClusterDev C, const int32_t* __restrict__ list, int co
     }
 }
 
+// Small fleets: a CTA of NW cooperating warps for every worker, in one launch
+// whatever the counts. A warp's build of 128 requests is a chain of about 9 us
+// and of 64 about 7; 4 and 2 warps take half of it, and with few workers it is
+// the chain that counts, not the work.
+template <int EW, int NW>
+__global__ void __launch_bounds__(NW * 32) k_build_few(DevParams P, ClusterDev C, PackSrc S)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int w = blockIdx.x;
+    if (S.off) {
+        if (threadIdx.x < 32) pack_worker(P, C, S, w);
+        __syncthreads();
+    }
+    if constexpr (NW == 1)
+        build_table<EW>(P, C, w, *reinterpret_cast<BuildSmem<EW, NW>*>(smraw));
+    else
+        build_table_fit<EW, NW>(P, C, w, C.n[w], smraw);
+}
+
 template <auto Kern>
 static cudaError_t allow_smem(size_t smem)
 {
@@ -136,6 +155,7 @@ static cudaError_t allow_smem(size_t smem)
 }
 
 constexpr int COOP_NW = 8;
+constexpr int FEW_WORKERS = 608;  // four CTAs an SM: every worker's build starts at once
 
 template <int E>
 static cudaError_t build_e(const DevParams& P, const ClusterDev& C, const int32_t* list, int count,
@@ -144,6 +164,13 @@ static cudaError_t build_e(const DevParams& P, const ClusterDev& C, const int32_
     if (count <= 0) return cudaSuccess;
     const int blocks = (count + BUILD_WARPS - 1) / BUILD_WARPS;
     cudaError_t e;
+    if (!list && count <= FEW_WORKERS) {
+        constexpr int NW = E < COOP_NW ? E : COOP_NW;
+        const size_t sf = sizeof(BuildSmem<E / NW, NW>);
+        if ((e = allow_smem<k_build_few<E / NW, NW>>(sf)) != cudaSuccess) return e;
+        k_build_few<E / NW, NW><<<count, NW * 32, sf, st>>>(P, C, S);
+        return cudaGetLastError();
+    }
     if constexpr (E > E_LO) {
         constexpr int EW = E / COOP_NW;
         const size_t sc = sizeof(BuildSmem<EW, COOP_NW>);
