@@ -58,6 +58,9 @@ cudaError_t launch_score(const DevParams& P, const ClusterDev& C, int n_cand, co
                          bool pend, cudaStream_t st, cudaEvent_t ev0 = nullptr,
                          cudaEvent_t ev1 = nullptr, bool prepared = false,
                          const int32_t* ranked = nullptr, int ld = 0);
+// Whether launch_score serves n candidates without sorting them (small calls:
+// it needs neither B nor launch_cand_prep). Not under the wait test hook.
+bool score_direct(const DevParams& P, const ClusterDev& C, int n);
 // The candidate preparation of launch_score alone (it reads no table): the
 // validated per-candidate records sorted by predicted output, and the
 // argbest keys reset. W is the cluster's worker count (output row stride).

@@ -563,9 +563,11 @@ int score_impl(aladdin_cluster* cl, int32_t n, const int32_t* in, const int32_t*
         (rc = stage_out(cl->s_kv, kv_peak, pairs, &dkv, &hk)) ||
         (rc = stage_out(cl->s_tc, t_cand, pairs, &dtc, &ht)))
         return rc;
-    CK(cl->sorted.ensure(sizeof(float4) * CAND_REC_F4 * C));
-    CK(cl->hist.ensure(sizeof(int32_t) * ((size_t)cl->hp.K + 2)));
-    CK(cl->best.ensure(sizeof(unsigned int) * C));
+    if (!score_direct(cl->dp, cl->dev, n)) {
+        CK(cl->sorted.ensure(sizeof(float4) * CAND_REC_F4 * C));
+        CK(cl->hist.ensure(sizeof(int32_t) * ((size_t)cl->hp.K + 2)));
+        CK(cl->best.ensure(sizeof(unsigned int) * C));
+    }
     ScoreBuffers B{cl->sorted.as<float4>(), cl->hist.as<int32_t>(), cl->best.as<unsigned int>()};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cl->timing && (dflags || dmargin || darg)) {
@@ -684,7 +686,13 @@ try {
     }
     if (!cand_in || !cand_pred) return ALADDIN_ERR_ARG;
     CK(cudaSetDevice(cl->device));
-    if (!cl->side) {
+    const int32_t* roff = static_cast<const int32_t*>(view[0]);
+    const int32_t* rin = static_cast<const int32_t*>(view[1]);
+    const int32_t* rgen = static_cast<const int32_t*>(view[2]);
+    const int32_t* rpred = static_cast<const int32_t*>(view[3]);
+    const float* rtdec = static_cast<const float*>(view[4]);
+    const bool small = score_direct(cl->dp, cl->dev, n_cand);  // nothing to overlap
+    if (!small && !cl->side) {
         CK(cudaStreamCreateWithFlags(&cl->side, cudaStreamNonBlocking));
         CK(cudaEventCreateWithFlags(&cl->ev_fork, cudaEventDisableTiming));
         CK(cudaEventCreateWithFlags(&cl->ev_join, cudaEventDisableTiming));
@@ -696,9 +704,11 @@ try {
     float* dm = static_cast<float*>(view[9]);
     int32_t* da = static_cast<int32_t*>(view[10]);
     const size_t C = (size_t)n_cand;
-    CK(cl->sorted.ensure(sizeof(float4) * CAND_REC_F4 * C));
-    CK(cl->hist.ensure(sizeof(int32_t) * ((size_t)cl->hp.K + 2)));
-    CK(cl->best.ensure(sizeof(unsigned int) * C));
+    if (!small) {
+        CK(cl->sorted.ensure(sizeof(float4) * CAND_REC_F4 * C));
+        CK(cl->hist.ensure(sizeof(int32_t) * ((size_t)cl->hp.K + 2)));
+        CK(cl->best.ensure(sizeof(unsigned int) * C));
+    }
     ScoreBuffers B{cl->sorted.as<float4>(), cl->hist.as<int32_t>(), cl->best.as<unsigned int>()};
     // fork: the candidates are sorted on the side stream (they read no table)
     // while the cluster's stream packs the state and builds the tables. The
@@ -706,10 +716,7 @@ try {
     // starts from the fork point recorded before it.
     auto enqueue_load = [&]() -> int {
         CK(cudaEventRecord(cl->ev_fork, cl->st));
-        const int r = load_requests_dev(
-            cl, static_cast<const int32_t*>(view[0]), static_cast<const int32_t*>(view[1]),
-            static_cast<const int32_t*>(view[2]), static_cast<const int32_t*>(view[3]),
-            static_cast<const float*>(view[4]));
+        const int r = load_requests_dev(cl, roff, rin, rgen, rpred, rtdec);
         CK(cudaStreamWaitEvent(cl->side, cl->ev_fork, 0));
         CK(launch_cand_prep(cl->dp, cl->W, n_cand, cin, cpr, cw, B, cl->side));
         CK(cudaEventRecord(cl->ev_join, cl->side));
@@ -731,7 +738,10 @@ try {
     // the cached graph alone
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(cl->st, &cap));
-    if (cap != cudaStreamCaptureStatusNone) {
+    if (small) {
+        rc = load_requests_dev(cl, roff, rin, rgen, rpred, rtdec);
+        if (rc) return rc;
+    } else if (cap != cudaStreamCaptureStatusNone) {
         rc = enqueue_load();
         if (rc) return rc;
     } else {

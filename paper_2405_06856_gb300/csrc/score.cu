@@ -603,6 +603,149 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32) k_score_scalar(ScoreArgs A)
     }
 }
 
+// Small calls: every pair on its own, without sorting the candidates. TW
+// threads take a candidate, each DIRECT_U workers at a time (the row searches
+// advance together: each is a chain of dependent loads, which is what bounds
+// the kernel), and the candidate's argbest is reduced and written in place.
+// One launch instead of six (histogram reset, count, scan, scatter, k_score,
+// k_finalize); the values are k_score's.
+constexpr int DIRECT_THREADS = 256;
+constexpr int DIRECT_U = 4;
+
+struct DirectArgs {
+    DevParams P;
+    ClusterDev C;
+    int n;
+    const int32_t* in;
+    const int32_t* pred;
+    const float* wait;
+    uint8_t* flags;
+    float* margin;
+    int32_t* argbest;
+    int tw;    // threads a candidate (32 .. DIRECT_THREADS)
+    int pend;  // some worker holds requests placed in an open round
+    const int32_t* order;  // nullptr, or rank order: output column k is worker order[k]
+    int ld;    // output row stride (elements)
+};
+
+__global__ void __launch_bounds__(DIRECT_THREADS) k_score_direct(DirectArgs A)
+{
+    __shared__ unsigned part[DIRECT_THREADS / 32];
+    const DevParams& P = A.P;
+    const ClusterDev& C = A.C;
+    const int W = C.W, tw = A.tw, lane = threadIdx.x & 31;
+    const int per = DIRECT_THREADS / tw, sub = threadIdx.x / tw, t = threadIdx.x - sub * tw;
+    const int c = blockIdx.x * per + sub;
+    unsigned best = 0xffffffffu;
+    bool valid = false;
+    if (c < A.n) {
+        const CandRec cr = make_cand(P, A.in[c], A.pred[c], A.wait ? A.wait[c] : 0.0f, c);
+        valid = cr.valid != 0;
+        const size_t row0 = (size_t)c * (size_t)A.ld;
+        for (int w0 = t; w0 < W; w0 += tw * DIRECT_U) {
+            int wk[DIRECT_U], lo[DIRECT_U], hi[DIRECT_U];
+#pragma unroll
+            for (int u = 0; u < DIRECT_U; ++u) {
+                const int col = w0 + u * tw;
+                const int k = col < W ? col : 0;
+                wk[u] = A.order ? __ldg(&A.order[k]) : k;
+                lo[u] = 0;
+                hi[u] = col < W && valid ? __ldg(&C.R[wk[u]]) : 0;
+            }
+            for (;;) {
+                bool more = false;
+                int nxt[DIRECT_U], mid[DIRECT_U];
+#pragma unroll
+                for (int u = 0; u < DIRECT_U; ++u) {
+                    mid[u] = (lo[u] + hi[u]) >> 1;
+                    nxt[u] = lo[u] < hi[u]
+                                 ? __float_as_int(__ldg(&C.tab[((long long)wk[u] * C.rows + mid[u]) * ROW_F4].x))
+                                 : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < DIRECT_U; ++u) {
+                    if (lo[u] >= hi[u]) continue;
+                    if (nxt[u] > cr.ri) hi[u] = mid[u];
+                    else lo[u] = mid[u] + 1;
+                    more |= lo[u] < hi[u];
+                }
+                if (!more) break;
+            }
+            Row r[DIRECT_U];
+            float2 ext[DIRECT_U];
+            float4 wr[DIRECT_U];
+            float2 wa[DIRECT_U];
+#pragma unroll
+            for (int u = 0; u < DIRECT_U; ++u) {
+                const long long row = (long long)wk[u] * C.rows + lo[u];
+                r[u] = load_row(C.tab, row);
+                ext[u] = A.pend ? __ldg(&C.tab2[row]) : make_float2(f_inf(), f_inf());
+                wr[u] = __ldg(&C.wrec[wk[u]]);
+                wa[u] = P.approx ? __ldg(&C.wapx[wk[u]]) : make_float2(0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int u = 0; u < DIRECT_U; ++u) {
+                const int col = w0 + u * tw;
+                if (col >= W) continue;
+                float m = __int_as_float(0x7fc00000);
+                unsigned f = 0x80u;
+                if (valid) {
+                    f = eval_pair_mode(P.approx != 0, r[u].v0, r[u].v1, ext[u], wr[u], wa[u], cr, m);
+                    if (f == 15u) best = min(best, (unsigned)__float_as_int(wr[u].w));
+                }
+                if (A.flags) A.flags[row0 + col] = (uint8_t)f;
+                if (A.margin) A.margin[row0 + col] = m;
+            }
+        }
+    }
+    if (!A.argbest) return;
+    best = __reduce_min_sync(FULL, best);
+    if (tw > 32) {
+        if (lane == 0) part[threadIdx.x >> 5] = best;
+        __syncthreads();
+        if (t == 0)
+            for (int k = 1; k < tw / 32; ++k) best = min(best, part[(threadIdx.x >> 5) + k]);
+    }
+    if (t == 0 && c < A.n)
+        A.argbest[c] = !valid ? -2 : best == 0xffffffffu ? -1 : C.order[best];
+}
+
+// Calls that k_score_direct serves: up to about a million pairs (there both
+// ways take the same time) on fleets whose row searches a CTA finishes in a
+// few steps.
+constexpr long long DIRECT_PAIRS = 1ll << 20;
+constexpr int DIRECT_MAX_W = 2048;
+
+bool score_direct(const DevParams& P, const ClusterDev& C, int n)
+{
+    return !P.wait_test && C.W <= DIRECT_MAX_W && (long long)C.W * n <= DIRECT_PAIRS;
+}
+
+static cudaError_t launch_direct(const DevParams& P, const ClusterDev& C, int n, const int32_t* in,
+                                 const int32_t* pred, const float* wait, uint8_t* flags,
+                                 float* margin, int32_t* argbest, bool pend, const int32_t* ranked,
+                                 int row, cudaStream_t st)
+{
+    DirectArgs A;
+    A.P = P;
+    A.C = C;
+    A.n = n;
+    A.in = in;
+    A.pred = pred;
+    A.wait = wait;
+    A.flags = flags;
+    A.margin = margin;
+    A.argbest = argbest;
+    A.tw = 32;
+    while (A.tw < DIRECT_THREADS && A.tw * DIRECT_U < C.W) A.tw *= 2;
+    A.pend = pend ? 1 : 0;
+    A.order = ranked;
+    A.ld = row;
+    const int per = DIRECT_THREADS / A.tw;
+    k_score_direct<<<(n + per - 1) / per, DIRECT_THREADS, 0, st>>>(A);
+    return cudaGetLastError();
+}
+
 template <int SLOTS, bool SF, bool SMG, bool ARG, bool PEND, bool FULLT, bool APPROX>
 static cudaError_t launch_vec(const ScoreArgs& A0, cudaStream_t st)
 {
@@ -764,7 +907,7 @@ cudaError_t prepare_score_kernels()
         (const void*)k_score_scalar<true, false, true>, (const void*)k_score_scalar<false, true, true>,
         (const void*)k_score_scalar<true, false, false>, (const void*)k_score_scalar<false, true, false>,
         (const void*)k_score_scalar<false, false, true>, (const void*)k_cand_count,
-        (const void*)k_scan_hist, (const void*)k_cand_scatter, (const void*)k_finalize,
+        (const void*)k_score_direct, (const void*)k_scan_hist, (const void*)k_cand_scatter, (const void*)k_finalize,
         (const void*)k_detail};
     for (const void* k : kerns)
         if ((e = cudaFuncGetAttributes(&fa, k)) != cudaSuccess) return e;
@@ -796,7 +939,12 @@ cudaError_t launch_score(const DevParams& P, const ClusterDev& C, int n, const i
     const int tb = 256, nb = (n + tb - 1) / tb;
     const bool need_score = flags || margin || argbest;
     const int row = ld > 0 ? ld : C.W;  // output row stride
-    if (need_score) {
+    if (need_score && score_direct(P, C, n)) {
+        if (ev0) cudaEventRecord(ev0, st);
+        e = launch_direct(P, C, n, in, pred, wait, flags, margin, argbest, pend, ranked, row, st);
+        if (e != cudaSuccess) return e;
+        if (ev1) cudaEventRecord(ev1, st);
+    } else if (need_score) {
         if (!prepared && (e = launch_cand_prep(P, row, n, in, pred, wait, B, st)) != cudaSuccess)
             return e;
 
