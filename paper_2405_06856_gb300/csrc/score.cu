@@ -18,7 +18,6 @@
 namespace aladdin {
 
 constexpr int SCORE_WARPS = 4;
-constexpr int SCORE_CHUNK = 256;
 
 __global__ void k_cand_count(DevParams P, int n, const int32_t* __restrict__ in,
                              const int32_t* __restrict__ pred, const float* __restrict__ wait,
@@ -85,12 +84,9 @@ struct ScoreArgs {
     uint8_t* flags;
     float* margin;
     unsigned int* best;
-    int tiles, chunks;
-    int approx;  // approximate-mode constraints (b) and (d)
     long long wait_limit;  // mbarrier polls before a wait gives up
     int withhold;          // test hook: the first candidate copy is not issued
     const int32_t* order;  // nullptr, or rank order: output column k is worker order[k]
-    int ld;                // output row stride (elements)
 };
 
 __global__ void k_cand_scatter(DevParams P, int n, int W, const int32_t* __restrict__ in,
@@ -267,10 +263,15 @@ __device__ __forceinline__ void take_row(Slot<PEND>& q, const Row& r, const floa
     }
 }
 
-// One CTA = SCORE_WARPS warps x 32 lanes x SLOTS consecutive workers and one
-// contiguous range of sorted candidates (one wave of CTAs, equal shares).
-// Requires W % 4 == 0 and 16-byte aligned outputs. PEND: some worker holds
-// requests placed in an open round (pending prefill and its TTFT/ATGT bounds).
+// One CTA = SCORE_WARPS warps x 32 lanes x SLOTS workers and one contiguous
+// range of sorted candidates (one wave of CTAs, equal shares). TILE: 1, a lane's
+// workers are consecutive and its outputs one vector store (W % 4 == 0 and
+// 16-byte aligned outputs); 2, and every lane holds workers; 0, neither: the
+// lane's workers are 32 apart, so that each slot's stores are one segment per
+// warp whatever the row's alignment (1,001 workers x 5,003 candidates 150 ->
+// 60 us against a warp per 32 workers that read the candidates from global
+// memory). PEND: some worker holds requests placed in an open round (pending
+// prefill and its TTFT/ATGT bounds).
 #ifndef ALADDIN_STORE_HINT
 #define ALADDIN_STORE_HINT 1
 #endif
@@ -284,7 +285,7 @@ __device__ __forceinline__ void st_out(T* p, T v)
 #endif
 }
 
-template <int SLOTS, bool SF, bool SMG, bool ARG, bool PEND, bool FULLT, bool APPROX>
+template <int SLOTS, bool SF, bool SMG, bool ARG, bool PEND, int TILE, bool APPROX>
 __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MINB) k_score(VecArgs A)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -311,9 +312,10 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MIN
     }
 
     const int wbase = (tile * SCORE_WARPS + warp) * 32 * SLOTS;
-    const int w0 = wbase + lane * SLOTS;
-    const bool live = FULLT || w0 < W;
-    const bool warp_live = FULLT || wbase < W;
+    const int w0 = TILE ? wbase + lane * SLOTS : wbase + lane;
+    constexpr int WS = TILE ? 1 : 32;  // between a lane's workers
+    const bool live = TILE == 2 || w0 < W;  // the lane's first worker exists
+    const bool warp_live = TILE == 2 || wbase < W;
     uint8_t* const fbase = SF ? A.flags + (live ? w0 : 0) : nullptr;
     float* const mbase = SMG ? A.margin + (live ? w0 : 0) : nullptr;
     const int last_row = A.C.rows - 1;
@@ -360,7 +362,9 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MIN
                 const int r_first = __float_as_int(cs[2].x);
 #pragma unroll
                 for (int s = 0; s < SLOTS; ++s) {
-                    wk[s] = live ? (A.order ? __ldg(&A.order[w0 + s]) : w0 + s) : W - 1;
+                    const int col = w0 + s * WS;
+                    const bool here = TILE == 2 || (TILE == 1 ? live : col < W);
+                    wk[s] = here ? (A.order ? __ldg(&A.order[col]) : col) : W - 1;
                     const long long rb = (long long)wk[s] * A.C.rows;
                     p[s] = find_row(A.C.tab, rb, __ldg(&A.C.R[wk[s]]), r_first);
                     const long long pn = rb + min(p[s] + 1, last_row);
@@ -376,7 +380,7 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MIN
                     inv_s[s] = wr.x;
                     nZO[s] = -wr.y;
                     ZW[s] = wr.z;
-                    rank[s] = live ? (unsigned)__float_as_int(wr.w) : 0xffffffffu;
+                    rank[s] = here ? (unsigned)__float_as_int(wr.w) : 0xffffffffu;
                     if constexpr (APPROX) {
                         const float2 wa = __ldg(&A.C.wapx[wk[s]]);
                         bd[s] = wa.x;
@@ -461,7 +465,15 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MIN
                             d[3][s] = ca;
                         }
                     }
-                    m[s] = fmin3(fminf(d[0][s], d[1][s]), d[2][s], d[3][s]);
+                    // without flags from the smallest bound less the prompt (rounding is
+                    // monotone: the same value as the smallest headroom, two operations fewer)
+                    if constexpr (!SF)
+                        m[s] = fminf(fmin3(APPROX ? fminf(t.kvB1, fmaf(r, t.np1n, t.kvE)) : xkv[s],
+                                           PEND ? fminf(tt, ZW[s]) : tt,
+                                           APPROX ? bd[s % (APPROX ? SLOTS : 1)] : xdt[s]) - a,
+                                     d[3][s]);
+                    else
+                        m[s] = fmin3(fminf(d[0][s], d[1][s]), d[2][s], d[3][s]);
                     if (ARG) kmin = min(kmin, (__float_as_uint(m[s]) & 0x80000000u) | rank[s]);
                 }
             };
@@ -470,15 +482,27 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MIN
                 const unsigned long long off = rec_off(i);
                 if (SF) {
                     const unsigned f = pack_flags<SLOTS>(d);
-                    if (SLOTS == 4) st_out(reinterpret_cast<unsigned int*>(fbase + off), f);
-                    else st_out(reinterpret_cast<unsigned short*>(fbase + off), (unsigned short)f);
+                    if (TILE == 0) {
+#pragma unroll
+                        for (int s = 0; s < SLOTS; ++s)
+                            if (w0 + s * WS < W) fbase[off + s * WS] = (uint8_t)(f >> (8 * s));
+                    } else if (SLOTS == 4) {
+                        st_out(reinterpret_cast<unsigned int*>(fbase + off), f);
+                    } else {
+                        st_out(reinterpret_cast<unsigned short*>(fbase + off), (unsigned short)f);
+                    }
                 }
                 if (SMG) {
-                    if (SLOTS == 4)
+                    if (TILE == 0) {
+#pragma unroll
+                        for (int s = 0; s < SLOTS; ++s)
+                            if (w0 + s * WS < W) st_out(mbase + off + s * WS, m[s]);
+                    } else if (SLOTS == 4) {
                         st_out(reinterpret_cast<float4*>(mbase + off),
                                make_float4(m[0], m[1], m[2 % SLOTS], m[3 % SLOTS]));
-                    else
+                    } else {
                         st_out(reinterpret_cast<float2*>(mbase + off), make_float2(m[0], m[1]));
+                    }
                 }
             };
             auto score_one = [&](int i) {
@@ -496,8 +520,9 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MIN
                     const unsigned long long off = rec_off(i);
 #pragma unroll
                     for (int s = 0; s < SLOTS; ++s) {
-                        if (SF) fbase[off + s] = 0x80;
-                        if (SMG) mbase[off + s] = __int_as_float(0x7fc00000);
+                        if (TILE == 0 && w0 + s * WS >= W) continue;
+                        if (SF) fbase[off + s * WS] = 0x80;
+                        if (SMG) mbase[off + s * WS] = __int_as_float(0x7fc00000);
                     }
                 }
                 if (ARG) kbase[i] = 0xffffffffu;
@@ -541,65 +566,6 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, PEND ? 3 : ALADDIN_SCORE_MIN
             }
         }
         __syncthreads();  // buffer `buf` and kmin are reused two chunks later
-    }
-}
-
-// Fallback for W % 4 != 0 or unaligned outputs: one worker per lane, scalar
-// stores, candidate records read from global memory.
-template <bool SF, bool SMG, bool ARG>
-__global__ void __launch_bounds__(SCORE_WARPS * 32) k_score_scalar(ScoreArgs A)
-{
-    const int lane = threadIdx.x & 31;
-    const int unit = blockIdx.x * SCORE_WARPS + (threadIdx.x >> 5);
-    if (unit >= A.tiles * A.chunks) return;
-    const int tile = unit % A.tiles, chunk = unit / A.tiles;
-    const int W = A.C.W;
-    const int w = tile * 32 + lane;  // output column
-    const bool live = w < W;
-    const int wc = live ? (A.order ? __ldg(&A.order[w]) : w) : W - 1;  // its worker
-    const int c0 = chunk * SCORE_CHUNK;
-    const int c1 = min(c0 + SCORE_CHUNK, A.n_cand);
-    const long long rb = (long long)wc * A.C.rows;
-    const int last_row = A.C.rows - 1;
-    const float4* recs = reinterpret_cast<const float4*>(A.cand);
-    int p = find_row(A.C.tab, rb, A.C.R[wc], __float_as_int(__ldg(&recs[(size_t)c0 * REC_F4 + 2].x)));
-    Row cur = load_row(A.C.tab, rb + p);
-    float2 ext = __ldg(&A.C.tab2[rb + p]);
-    const float4 wr = __ldg(&A.C.wrec[wc]);
-    const float2 wa = A.approx ? __ldg(&A.C.wapx[wc]) : make_float2(0.0f, 0.0f);
-    const unsigned rank = live ? (unsigned)__float_as_int(wr.w) : 0xffffffffu;
-    for (int c = c0; c < c1; ++c) {
-        const float4* cp = recs + (size_t)c * REC_F4;
-        const float4 q0 = __ldg(cp), q1 = __ldg(cp + 1), q2 = __ldg(cp + 2);
-        CandRec cr;
-        cr.a = q0.x; cr.r = q0.y; cr.inv_r = q0.z; cr.Ua = q0.w;
-        cr.inv_d1 = q1.x; cr.nXd1 = q1.y; cr.inv_d2 = q1.z; cr.Zc = q1.w;
-        cr.ri = __float_as_int(q2.x);
-        cr.orig = __float_as_int(q2.y);
-        const size_t off = (size_t)cr.orig * (size_t)A.ld + (size_t)w;
-        if (cr.ri == 0) {
-            if (live) {
-                if (SF) A.flags[off] = 0x80;
-                if (SMG) A.margin[off] = __int_as_float(0x7fc00000);
-            }
-            continue;
-        }
-        while (cr.ri >= __float_as_int(cur.v0.x) && p < last_row) {
-            p += 1;
-            cur = load_row(A.C.tab, rb + p);
-            ext = __ldg(&A.C.tab2[rb + p]);
-        }
-        float m;
-        const unsigned f = eval_pair_mode(A.approx != 0, cur.v0, cur.v1, ext, wr, wa, cr, m);
-        if (live) {
-            if (SF) A.flags[off] = (uint8_t)f;
-            if (SMG) __stcs(A.margin + off, m);
-        }
-        if (ARG) {
-            unsigned kmin = (f == 15u) ? rank : 0xffffffffu;
-            kmin = __reduce_min_sync(FULL, kmin);
-            if (lane == 0 && kmin != 0xffffffffu) atomicMin(A.best + cr.orig, kmin);
-        }
     }
 }
 
@@ -746,7 +712,7 @@ static cudaError_t launch_direct(const DevParams& P, const ClusterDev& C, int n,
     return cudaGetLastError();
 }
 
-template <int SLOTS, bool SF, bool SMG, bool ARG, bool PEND, bool FULLT, bool APPROX>
+template <int SLOTS, bool SF, bool SMG, bool ARG, bool PEND, int TILE, bool APPROX>
 static cudaError_t launch_vec(const ScoreArgs& A0, cudaStream_t st)
 {
     VecArgs A;
@@ -765,7 +731,7 @@ static cudaError_t launch_vec(const ScoreArgs& A0, cudaStream_t st)
     cudaError_t e = device_info(&d);
     if (e != cudaSuccess) return e;
     int per_sm = 0;  // occupancy of this instantiation on this device (cached)
-    e = kernel_occupancy<k_score<SLOTS, SF, SMG, ARG, PEND, FULLT, APPROX>>(SCORE_WARPS * 32, smem,
+    e = kernel_occupancy<k_score<SLOTS, SF, SMG, ARG, PEND, TILE, APPROX>>(SCORE_WARPS * 32, smem,
                                                                           &per_sm);
     if (e != cudaSuccess) return e;
     // one wave: per_tile CTAs share each worker tile's candidates equally
@@ -775,45 +741,45 @@ static cudaError_t launch_vec(const ScoreArgs& A0, cudaStream_t st)
     const int max_parts = (A.n_cand + 63) / 64;  // at least 64 candidates per CTA
     if (per_tile > max_parts) per_tile = max_parts;
     A.per_tile = per_tile;
-    k_score<SLOTS, SF, SMG, ARG, PEND, FULLT, APPROX><<<A.tiles * per_tile, SCORE_WARPS * 32, smem, st>>>(A);
+    k_score<SLOTS, SF, SMG, ARG, PEND, TILE, APPROX><<<A.tiles * per_tile, SCORE_WARPS * 32, smem, st>>>(A);
     return cudaGetLastError();
 }
 
-template <bool PEND, bool FULLT, bool APPROX>
+template <bool PEND, int TILE, bool APPROX>
 static cudaError_t dispatch_vec3(bool sf, bool smg, bool arg, const ScoreArgs& A, cudaStream_t st)
 {
     constexpr int S = ALADDIN_SCORE_SLOTS;
-    if (sf && smg && arg) return launch_vec<S, true, true, true, PEND, FULLT, APPROX>(A, st);
-    if (sf && smg) return launch_vec<S, true, true, false, PEND, FULLT, APPROX>(A, st);
-    if (sf && arg) return launch_vec<S, true, false, true, PEND, FULLT, APPROX>(A, st);
-    if (smg && arg) return launch_vec<S, false, true, true, PEND, FULLT, APPROX>(A, st);
-    if (sf) return launch_vec<S, true, false, false, PEND, FULLT, APPROX>(A, st);
-    if (smg) return launch_vec<S, false, true, false, PEND, FULLT, APPROX>(A, st);
-    return launch_vec<S, false, false, true, PEND, FULLT, APPROX>(A, st);
+    if (sf && smg && arg) return launch_vec<S, true, true, true, PEND, TILE, APPROX>(A, st);
+    if (sf && smg) return launch_vec<S, true, true, false, PEND, TILE, APPROX>(A, st);
+    if (sf && arg) return launch_vec<S, true, false, true, PEND, TILE, APPROX>(A, st);
+    if (smg && arg) return launch_vec<S, false, true, true, PEND, TILE, APPROX>(A, st);
+    if (sf) return launch_vec<S, true, false, false, PEND, TILE, APPROX>(A, st);
+    if (smg) return launch_vec<S, false, true, false, PEND, TILE, APPROX>(A, st);
+    return launch_vec<S, false, false, true, PEND, TILE, APPROX>(A, st);
 }
 
-template <bool PEND, bool FULLT>
+template <bool PEND, int TILE>
 static cudaError_t dispatch_vec2(bool approx, bool sf, bool smg, bool arg, const ScoreArgs& A,
                                  cudaStream_t st)
 {
-    return approx ? dispatch_vec3<PEND, FULLT, true>(sf, smg, arg, A, st)
-                  : dispatch_vec3<PEND, FULLT, false>(sf, smg, arg, A, st);
+    return approx ? dispatch_vec3<PEND, TILE, true>(sf, smg, arg, A, st)
+                  : dispatch_vec3<PEND, TILE, false>(sf, smg, arg, A, st);
 }
 
 template <bool PEND>
-static cudaError_t dispatch_vec(bool approx, bool sf, bool smg, bool arg, const ScoreArgs& A,
-                                cudaStream_t st)
+static cudaError_t dispatch_vec(bool vec, bool approx, bool sf, bool smg, bool arg,
+                                const ScoreArgs& A, cudaStream_t st)
 {
     // every lane of every CTA tile holds a worker: no per-lane predicate
     const bool full = A.C.W % (SCORE_WARPS * 32 * ALADDIN_SCORE_SLOTS) == 0;
-    return full ? dispatch_vec2<PEND, true>(approx, sf, smg, arg, A, st)
-                : dispatch_vec2<PEND, false>(approx, sf, smg, arg, A, st);
+    if (!vec) return dispatch_vec2<PEND, 0>(approx, sf, smg, arg, A, st);
+    return full ? dispatch_vec2<PEND, 2>(approx, sf, smg, arg, A, st)
+                : dispatch_vec2<PEND, 1>(approx, sf, smg, arg, A, st);
 }
 
 // prepare_score_kernels: every k_score instantiation dispatch_vec can reach
-// (seven output combinations x pending x full tile x approximate), the scalar
-// variants and the candidate preparation, finalize and detail kernels.
-template <bool PEND, bool FULLT, bool APPROX>
+// (seven output combinations x pending x tile kind x approximate) and the candidate preparation, finalize and detail kernels.
+template <bool PEND, int TILE, bool APPROX>
 static cudaError_t prepare_vec3()
 {
     constexpr int S = ALADDIN_SCORE_SLOTS;
@@ -821,24 +787,15 @@ static cudaError_t prepare_vec3()
     constexpr size_t M = sizeof(ScoreSmem);
     int ps = 0;
     cudaError_t e;
-    if ((e = kernel_occupancy<k_score<S, true, true, true, PEND, FULLT, APPROX>>(T, M, &ps)) ||
-        (e = kernel_occupancy<k_score<S, true, true, false, PEND, FULLT, APPROX>>(T, M, &ps)) ||
-        (e = kernel_occupancy<k_score<S, true, false, true, PEND, FULLT, APPROX>>(T, M, &ps)) ||
-        (e = kernel_occupancy<k_score<S, false, true, true, PEND, FULLT, APPROX>>(T, M, &ps)) ||
-        (e = kernel_occupancy<k_score<S, true, false, false, PEND, FULLT, APPROX>>(T, M, &ps)) ||
-        (e = kernel_occupancy<k_score<S, false, true, false, PEND, FULLT, APPROX>>(T, M, &ps)) ||
-        (e = kernel_occupancy<k_score<S, false, false, true, PEND, FULLT, APPROX>>(T, M, &ps)))
+    if ((e = kernel_occupancy<k_score<S, true, true, true, PEND, TILE, APPROX>>(T, M, &ps)) ||
+        (e = kernel_occupancy<k_score<S, true, true, false, PEND, TILE, APPROX>>(T, M, &ps)) ||
+        (e = kernel_occupancy<k_score<S, true, false, true, PEND, TILE, APPROX>>(T, M, &ps)) ||
+        (e = kernel_occupancy<k_score<S, false, true, true, PEND, TILE, APPROX>>(T, M, &ps)) ||
+        (e = kernel_occupancy<k_score<S, true, false, false, PEND, TILE, APPROX>>(T, M, &ps)) ||
+        (e = kernel_occupancy<k_score<S, false, true, false, PEND, TILE, APPROX>>(T, M, &ps)) ||
+        (e = kernel_occupancy<k_score<S, false, false, true, PEND, TILE, APPROX>>(T, M, &ps)))
         return e;
     return cudaSuccess;
-}
-
-template <bool SF, bool SMG, bool ARG>
-static void launch_scalar(const ScoreArgs& A0, cudaStream_t st)
-{
-    ScoreArgs A = A0;
-    A.tiles = (A.C.W + 31) / 32;
-    const int units = A.tiles * A.chunks;
-    k_score_scalar<SF, SMG, ARG><<<(units + SCORE_WARPS - 1) / SCORE_WARPS, SCORE_WARPS * 32, 0, st>>>(A);
 }
 
 __global__ void k_finalize(DevParams P, int n, const int32_t* __restrict__ in,
@@ -896,17 +853,16 @@ __global__ void k_detail(DevParams P, ClusterDev C, int n, const int32_t* __rest
 cudaError_t prepare_score_kernels()
 {
     cudaError_t e;
-    if ((e = prepare_vec3<false, false, false>()) || (e = prepare_vec3<false, false, true>()) ||
-        (e = prepare_vec3<false, true, false>()) || (e = prepare_vec3<false, true, true>()) ||
-        (e = prepare_vec3<true, false, false>()) || (e = prepare_vec3<true, false, true>()) ||
-        (e = prepare_vec3<true, true, false>()) || (e = prepare_vec3<true, true, true>()))
+    if ((e = prepare_vec3<false, 0, false>()) || (e = prepare_vec3<false, 0, true>()) ||
+        (e = prepare_vec3<false, 1, false>()) || (e = prepare_vec3<false, 1, true>()) ||
+        (e = prepare_vec3<false, 2, false>()) || (e = prepare_vec3<false, 2, true>()) ||
+        (e = prepare_vec3<true, 0, false>()) || (e = prepare_vec3<true, 0, true>()) ||
+        (e = prepare_vec3<true, 1, false>()) || (e = prepare_vec3<true, 1, true>()) ||
+        (e = prepare_vec3<true, 2, false>()) || (e = prepare_vec3<true, 2, true>()))
         return e;
     cudaFuncAttributes fa;
     const void* kerns[] = {
-        (const void*)k_score_scalar<true, true, true>, (const void*)k_score_scalar<true, true, false>,
-        (const void*)k_score_scalar<true, false, true>, (const void*)k_score_scalar<false, true, true>,
-        (const void*)k_score_scalar<true, false, false>, (const void*)k_score_scalar<false, true, false>,
-        (const void*)k_score_scalar<false, false, true>, (const void*)k_cand_count,
+        (const void*)k_cand_count,
         (const void*)k_score_direct, (const void*)k_scan_hist, (const void*)k_cand_scatter, (const void*)k_finalize,
         (const void*)k_detail};
     for (const void* k : kerns)
@@ -955,31 +911,17 @@ cudaError_t launch_score(const DevParams& P, const ClusterDev& C, int n, const i
         A.flags = flags;
         A.margin = margin;
         A.best = argbest ? B.best : nullptr;
-        A.chunks = (n + SCORE_CHUNK - 1) / SCORE_CHUNK;
-        A.tiles = 0;
-        A.approx = P.approx;
         A.wait_limit = P.mbar_wait_limit;
         A.withhold = P.wait_test;
         A.order = ranked;
-        A.ld = row;
         if (ev0) cudaEventRecord(ev0, st);
         const bool vec = (C.W % 4 == 0) && (row % 4 == 0) && (((uintptr_t)flags & 3) == 0) &&
                          (((uintptr_t)margin & 15) == 0);
         const bool sf = flags != nullptr, smg = margin != nullptr, arg = argbest != nullptr;
-        if (vec) {
-            const bool ap = P.approx != 0;
-            e = pend ? dispatch_vec<true>(ap, sf, smg, arg, A, st)
-                     : dispatch_vec<false>(ap, sf, smg, arg, A, st);
-            if (e != cudaSuccess) return e;
-        } else {
-            if (sf && smg && arg) launch_scalar<true, true, true>(A, st);
-            else if (sf && smg) launch_scalar<true, true, false>(A, st);
-            else if (sf && arg) launch_scalar<true, false, true>(A, st);
-            else if (smg && arg) launch_scalar<false, true, true>(A, st);
-            else if (sf) launch_scalar<true, false, false>(A, st);
-            else if (smg) launch_scalar<false, true, false>(A, st);
-            else launch_scalar<false, false, true>(A, st);
-        }
+        const bool ap = P.approx != 0;
+        e = pend ? dispatch_vec<true>(vec, ap, sf, smg, arg, A, st)
+                 : dispatch_vec<false>(vec, ap, sf, smg, arg, A, st);
+        if (e != cudaSuccess) return e;
         if (ev1) cudaEventRecord(ev1, st);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
