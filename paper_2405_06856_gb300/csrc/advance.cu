@@ -32,7 +32,7 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* addr, doub
 template <int E>
 __global__ void __launch_bounds__(ADV_WARPS * 32)
 k_advance(DevParams P, ClusterDev C, double t_now, double dt, unsigned long long* stats,
-          const int* halt, unsigned long long* fail)
+          const int* halt, unsigned long long* fail, int exact)
 {
     if (halt && *halt != 0) return;
     const int lane = threadIdx.x & 31;
@@ -57,11 +57,11 @@ k_advance(DevParams P, ClusterDev C, double t_now, double dt, unsigned long long
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int x = e * 32 + lane;
-        if (x < n) alive |= 1u << e;
         in[e] = gen[e] = 0;
         evt[e] = 1;
         tdec[e] = 0.0;
         if (x < n) {
+            alive |= 1u << e;
             const long long slot = base + x;
             in[e] = C.in[slot];
             gen[e] = C.gen[slot];
@@ -108,27 +108,32 @@ k_advance(DevParams P, ClusterDev C, double t_now, double dt, unsigned long long
     // request, so at most max(real) iterations run).
     for (;;) {
         int b = 0;
-        long long K = 0;
+        int K = 0;  // a lane's share: at most 32 requests of 65,536 tokens
 #pragma unroll
-        for (int e = 0; e < E; ++e)
+        for (int e = 0; e < E; ++e) {
+            if (e * 32 >= n) break;  // uniform: a worker holds far fewer than its slots
             if ((alive >> e) & 1u) {
                 b += 1;
-                K += (long long)in[e] + gen[e] + 1;
+                K += in[e] + gen[e] + 1;
             }
-        b = warp_reduce(b, OpAdd<int>());
-        K = warp_reduce(K, OpAdd<long long>());
+        }
+        b = __reduce_add_sync(FULL, b);
+        K = __reduce_add_sync(FULL, K);  // at most 2^26
         if (b == 0 || !(start < t_end)) break;
         vkv += (long long)P.h * K + (long long)P.j * b > Mw ? 1 : 0;
         const double t = __dmul_rn(
             s, __dadd_rn(__dadd_rn(P.c3d, __dmul_rn(P.c2d, (double)b)), __dmul_rn(P.k2d, (double)K)));
 #pragma unroll
-        for (int e = 0; e < E; ++e)
+        for (int e = 0; e < E; ++e) {
+            if (e * 32 >= n) break;
             if ((alive >> e) & 1u) {
                 gen[e] += 1;
                 tdec[e] = __dadd_rn(tdec[e], t);
                 if (gen[e] >= evt[e]) {
                     const long long slot = base + e * 32 + lane;
-                    const int pr = C.pred[slot], rl = C.real[slot];
+                    // with exact predictions the event is the end
+                    const int pr = exact ? evt[e] : C.pred[slot];
+                    const int rl = exact ? evt[e] : C.real[slot];
                     if (gen[e] >= rl) {
                         if (rl < pr) {  // finished before its prediction
                             le_acc += rl - pr;
@@ -152,12 +157,14 @@ k_advance(DevParams P, ClusterDev C, double t_now, double dt, unsigned long long
                     }
                 }
             }
+        }
         start = __dadd_rn(start, t);
     }
     // Write the surviving requests back in their order, densely.
     int pos = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
+        if (e * 32 >= n) break;
         const unsigned bal = __ballot_sync(FULL, (alive >> e) & 1u);
         const int before = __popc(bal & ((1u << lane) - 1u));
         const long long src = base + e * 32 + lane;
@@ -220,24 +227,24 @@ k_advance(DevParams P, ClusterDev C, double t_now, double dt, unsigned long long
 template <int E>
 static cudaError_t advance_e(const DevParams& P, const ClusterDev& C, double t_now, double dt,
                              unsigned long long* stats, const int* halt, unsigned long long* fail,
-                             cudaStream_t st)
+                             bool exact, cudaStream_t st)
 {
     const int blocks = (C.W + ADV_WARPS - 1) / ADV_WARPS;
-    k_advance<E><<<blocks, ADV_WARPS * 32, 0, st>>>(P, C, t_now, dt, stats, halt, fail);
+    k_advance<E><<<blocks, ADV_WARPS * 32, 0, st>>>(P, C, t_now, dt, stats, halt, fail, exact ? 1 : 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_advance(const DevParams& P, const ClusterDev& C, double t_now, double dt,
                            unsigned long long* stats, const int* halt, cudaStream_t st,
-                           unsigned long long* fail)
+                           unsigned long long* fail, bool exact)
 {
     switch (lanes_per_worker(C.cap)) {
-    case 1: return advance_e<1>(P, C, t_now, dt, stats, halt, fail, st);
-    case 2: return advance_e<2>(P, C, t_now, dt, stats, halt, fail, st);
-    case 4: return advance_e<4>(P, C, t_now, dt, stats, halt, fail, st);
-    case 8: return advance_e<8>(P, C, t_now, dt, stats, halt, fail, st);
-    case 16: return advance_e<16>(P, C, t_now, dt, stats, halt, fail, st);
-    case 32: return advance_e<32>(P, C, t_now, dt, stats, halt, fail, st);
+    case 1: return advance_e<1>(P, C, t_now, dt, stats, halt, fail, exact, st);
+    case 2: return advance_e<2>(P, C, t_now, dt, stats, halt, fail, exact, st);
+    case 4: return advance_e<4>(P, C, t_now, dt, stats, halt, fail, exact, st);
+    case 8: return advance_e<8>(P, C, t_now, dt, stats, halt, fail, exact, st);
+    case 16: return advance_e<16>(P, C, t_now, dt, stats, halt, fail, exact, st);
+    case 32: return advance_e<32>(P, C, t_now, dt, stats, halt, fail, exact, st);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -208,11 +208,12 @@ cudaError_t prepare_score_kernels();
 // events [7] re-predictions, [8] early finishes. halt (device, nullable):
 // nothing runs when *halt != 0. fail (device, nullable): every violation is
 // also added to it (the simulation's failure counter). Each worker's error
-// events are added to C.le / C.be.
+// events are added to C.le / C.be. exact: every real length equals its
+// prediction, so that reaching it is the end (no such event).
 constexpr int STATS_N = 9;
 cudaError_t launch_advance(const DevParams& P, const ClusterDev& C, double t_now, double dt,
                            unsigned long long* stats, const int* halt, cudaStream_t st,
-                           unsigned long long* fail = nullptr);
+                           unsigned long long* fail = nullptr, bool exact = false);
 
 // A best-fit round of a placement call under grouped scheduling (P.groups >
 // 1, direct mode): one CTA per group, the groups in parallel. A group whose

@@ -969,6 +969,8 @@ int aladdin_cluster_advance(aladdin_cluster* cl, double dt_ms, double* stats)
 try {
     if (!cl || !(std::isfinite(dt_ms) && dt_ms >= 0)) return ALADDIN_ERR_ARG;
     CK(cudaSetDevice(cl->device));
+    // a cluster built by this API holds exact predictions, unless a checkpoint
+    // brought others
     CK(launch_advance(cl->dp, cl->dev, cl->t_now, dt_ms, cl->d_stats, nullptr, cl->st));
     cl->t_now += dt_ms;
     cl->round_open = false;
@@ -1390,7 +1392,8 @@ int simulate_impl(const aladdin_params& p, const aladdin_worker_cfg& cfg, int32_
         }
         next = end;
         // realized violations count as failures (counters[0])
-        CK(launch_advance(cl.dp, cl.dev, t, H, cl.d_stats, cl.d_status, st, counters));
+        CK(launch_advance(cl.dp, cl.dev, t, H, cl.d_stats, cl.d_status, st, counters,
+                          tr.real == nullptr));
         // JSQ and power of two read no table
         if (bestfit) CK(launch_build(cl.dp, cl.dev, nullptr, cl.W, st));
         hb++;
