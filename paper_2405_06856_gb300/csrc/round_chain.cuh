@@ -178,6 +178,7 @@ struct ChSmem {
     float tf[4][32];                 // and bounds
     int code[2], next[2];            // [run parity]
     int miss_w, miss_f, victim;
+    int left_n;                      // requests of the worker that left last
     int abort;
     int cnt[CH_WARPS + 1];
     int lq[CH_SCAN][64];             // look-ahead: slots to evaluate
@@ -996,8 +997,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         sm.ne[par][slot][ver] = new_elem(t, rw.x, rw.y);
     };
 
-    // CH_DECIDE: the outcomes of candidates [k0, k1), at most 32, logged by
-    // the links, written a lane each.
+    // The last look-ahead warp: the outcomes of candidates [k0, k1), at most 32,
+    // logged by the links, written a lane each.
     unsigned long long placed = 0, failed = 0;  // trace mode (the same in every lane)
     int keep = 0;                               // trace mode: waiting list
     auto flush = [&](int k0, int k1) CH_INLINE {
@@ -1241,7 +1242,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             mR[m] = R;
             mwrec[m] = wr;
             mkey[m] = kq;
-            mn[m] = n;
+            sm.left_n = n;
         }
         hot_group_sync<NWG>();  // the scratch is free
     };
@@ -1358,12 +1359,6 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                     C.n[w] = n0 + 1;
                     sm.ln[b] = n0;
                     sm.hn[v] = n0;
-                    mn[m] = (n0 + 1) | (int)0x80000000;
-                    if (f & CH_UNMOD) {
-                        mw[m] = w;
-                        const int pos = f & CH_IDX;
-                        modbits[pos >> 5] |= 1u << (pos & 31);
-                    }
                     own.m = m;
                     own.n += 1;
                     own.sumP += rw.x;
@@ -1469,8 +1464,6 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             const unsigned lru = __reduce_min_sync(
                 FULL, lane < KH ? ((unsigned)(hk_last + 1) << 4) | (unsigned)lane : 0xffffffffu);
             const int b = k & (CH_RING - 1);
-            __syncwarp();
-            flush(c, k);
             if (lane < KH) {
                 sm.hw[lane] = hk_w;
                 sm.hm[lane] = hk_m;
@@ -1480,9 +1473,21 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 sm.code[rp] = code;
                 sm.next[rp] = k;
                 if (code == CH_MISS) {
-                    sm.miss_w = sm.alt_w[b];
-                    sm.miss_f = sm.alt_f[b];
+                    const int w = sm.alt_w[b], f = sm.alt_f[b];
+                    sm.miss_w = w;
+                    sm.miss_f = f;
                     sm.victim = (int)(lru & 15u);
+                    // hot from here on (bit 31), so that the look-ahead leaves
+                    // it out
+                    if (!(f & CH_UNMOD)) {
+                        mn[f & CH_IDX] = (int)0x80000000;
+                    } else if (mcount < mmax) {
+                        const int pos = f & CH_IDX;
+                        mw[mcount] = w;
+                        mn[mcount] = (int)0x80000000;
+                        modbits[pos >> 5] |= 1u << (pos & 31);
+                    }
+                    sm.lw_[b] = w;
                 } else if (code == CH_STOP) {
                     *io.status = -2;  // ALADDIN_ERR_CAPACITY
                     if (!sim)
@@ -1498,17 +1503,10 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             }
             if (code == CH_STOP) break;
             const int f = sm.miss_f, v = sm.victim;
-            if ((f & CH_UNMOD) && mcount == mmax) {
-                stop_at = c;
-                break;
-            }
+            if ((f & CH_UNMOD) && mcount == mmax) break;
             if (f & CH_UNMOD) mcount++;
-            if (lane == 0) {
-                sm.lw_[c & (CH_RING - 1)] = sm.miss_w;
-                sm.abort = 0;
-            }
+            if (lane == 0) sm.abort = 0;
             cta_sync();
-            flush(c, c + 1);  // the slot it went to is known now
             if (lane == v) {
                 const ChOwn& o = sm.own[v];
                 hk_w = o.w;
@@ -1588,16 +1586,25 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         }
         if (!(lane & 1) && lane >> 1 < KH) sm.own[lane >> 1] = o;
     } else {
+        const bool clerk = warp == CH_WARPS - 1;  // fetches the records, writes the outcomes
+        bool primed = false;  // the first candidates were looked at during the last miss
+        int written = 0;      // candidates whose outcomes are written
         for (int rp = 0; c < n_cand; rp ^= 1) {
             if (alt_end <= c) {
-                for (int k = c + warp - CH_LOOK0; k < min(c + CH_SCAN, n_cand); k += CH_SCAN) look(k);
                 alt_end = min(c + CH_SCAN, n_cand);
+                const int k = c + warp - CH_LOOK0;
+                if (!primed && k < alt_end) look(k);
+                primed = false;
                 cta_sync();
             }
             const int new_end = min(alt_end + CH_AHEAD, n_cand);
             const int rec_new = max(rec_end, min(n_cand, new_end + CH_AHEAD));
-            if (warp == CH_WARPS - 1)
+            if (clerk) {
+                flush(written, c);  // (their records are in the ring until fetch takes their place)
+                written = c;
+                __syncwarp();
                 for (int k = rec_end + lane; k < rec_new; k += 32) fetch(k);
+            }
             if (A.F)
                 for (int k = rec_end + warp - CH_LOOK0; k < rec_new; k += CH_SCAN) fetch_row(k);
             rec_end = rec_new;
@@ -1613,17 +1620,65 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 continue;
             }
             if (code == CH_STOP) break;
-            const int f = sm.miss_f, v = sm.victim;
-            if ((f & CH_UNMOD) && mcount == mmax) break;
+            const int f = sm.miss_f, v = sm.victim, w = sm.miss_w;
+            if ((f & CH_UNMOD) && mcount == mmax) {
+                stop_at = c;
+                break;
+            }
             if (f & CH_UNMOD) mcount++;
-            cta_sync();
+            // while the hot warps write the leaving worker's table and load w:
+            // w's requests towards L1, and the next candidates looked at among
+            // the workers other than the leaving one
+            {
+                const int nw = C.n[w];
+                const long long base = (long long)w * cap;
+                for (int x = 32 * ((warp - CH_LOOK0) * 32 + lane); x < nw; x += 32 * 32 * CH_SCAN) {
+                    const void* const line[] = {C.skey + base + x, C.in + base + x,
+                                                C.gen + base + x, C.pred + base + x,
+                                                C.bank + base + x, C.pend + base + x};
+#pragma unroll
+                    for (int i = 0; i < 6; ++i)
+                        asm volatile("prefetch.global.L1 [%0];" ::"l"(line[i]));
+                }
+            }
             c += 1;
+            const int k = c + warp - CH_LOOK0;
+            if (k < n_cand) look(k);
+            cta_sync();
+            if (sm.hw[v] != NONE) {  // now the one that left
+                const int i = sm.hm[v], n = sm.left_n, b = k & (CH_RING - 1);
+                if (k < n_cand) {
+                    const CandRec cq = sm.rec[b];
+                    const int ow = mw[i];
+                    const unsigned long long ok = mkey[i];
+                    if (cq.valid && (sm.alt_w[b] == NONE || ok > sm.alt_k[b] ||
+                                     (ok == sm.alt_k[b] && ow < sm.alt_w[b])) &&
+                        (!filter || ow % GP == sm.raw[b].w)) {
+                        const long long rb = (long long)ow * C.rows;
+                        const long long row = rb + slot_row(i, rb, mR[i], cq.ri);
+                        const float4* t = C.tab + row * ROW_F4;
+                        float m;
+                        const unsigned fl =
+                            eval_pair_mode(P.approx != 0, t[0], t[1], C.tab2[row], mwrec[i],
+                                           P.approx ? C.wapx[ow] : make_float2(0.0f, 0.0f), cq, m);
+                        __syncwarp();
+                        if (fl == 15u && lane == 0) {
+                            sm.alt_k[b] = ok;
+                            sm.alt_w[b] = ow;
+                            sm.alt_f[b] = i | (n >= cap ? CH_FULL : 0);
+                        }
+                    }
+                }
+                if (warp == CH_LOOK0 && lane == 0) mn[i] = n;  // not hot any more
+            }
+            primed = true;
             alt_end = c;
         }
+        if (clerk) flush(written, c);
     }
     if (last_tables && warp >= CH_HOT)
         for (int k = 0; k <= KH; ++k) cta_sync();
-    if (warp == CH_DECIDE && lane == 0) {
+    if (warp == CH_WARPS - 1 && lane == 0) {
         if (!sim) {
             if (A.c_stop) *A.c_stop = stop_at;
         } else {
