@@ -85,6 +85,7 @@ struct ChCfg {
     static constexpr int NWG = 4;
     static constexpr int EPL = E / NWG;
     static constexpr int KH = CH_HOT / NWG;
+    static constexpr bool STAGE = EPL <= 4;  // look-ahead warps load the next hot worker
 };
 
 // Round-start entry of a rank position: the worker there, its key and count.
@@ -174,7 +175,14 @@ struct ChSmem {
     int ea[32 * E], ekv[32 * E], eSb[32 * E];
     long long eSK[32 * E];
     float ebnd[32 * E], esg[32 * E];
-    int ti[4][32];                   // its chunks' totals: rows, KV peaks, context
+    // a worker that becomes hot, formed by look-ahead warps while the hot ones
+    // write the leaving worker's table (bit 31 of sta: placed in this round)
+    static constexpr int ST = Cfg::STAGE ? 32 * E : 1;
+    int str[ST], sta[ST], stS[ST], stk[ST];
+    long long stK[ST];
+    float stb[ST], sty[ST], std_[ST];
+    ChOwn sto;
+    int ti[4][32];                   // a leaving worker's chunks' totals: rows, KV peaks, context
     float tf[4][32];                 // and bounds
     int code[2], next[2];            // [run parity]
     int miss_w, miss_f, victim;
@@ -210,6 +218,23 @@ template <int N>
 __device__ __forceinline__ void hot_group_sync()
 {
     asm volatile("bar.sync 4, %0;" ::"r"(N * 32) : "memory");
+}
+
+// The warps that stage a worker among themselves, and its handing over.
+template <int N>
+__device__ __forceinline__ void stage_group_sync()
+{
+    asm volatile("bar.sync 6, %0;" ::"r"(N * 32) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void staged_arrive()
+{
+    asm volatile("bar.arrive 7, %0;" ::"r"(2 * N * 32) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void staged_wait()
+{
+    asm volatile("bar.sync 7, %0;" ::"r"(2 * N * 32) : "memory");
 }
 
 // A link's two barriers: votes and terms are in (hot warps, CH_DECIDE and
@@ -666,7 +691,11 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         }
         return t;
     };
-    // load worker w's requests into this slot's warps
+    // load worker w's requests into the registers of NWG warps
+    auto group_sync = [&]() CH_INLINE {
+        if constexpr (Cfg::STAGE) stage_group_sync<NWG>();
+        else hot_group_sync<NWG>();
+    };
     auto load = [&](Hot<EPL>& H, ChOwn& own, int w) CH_INLINE {
         const long long base = (long long)w * cap;
         const int n = C.n[w];
@@ -759,7 +788,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             sm.lw[q] = wp;
             sm.lm[q] = dm;
         }
-        hot_group_sync<NWG>();
+        group_sync();
         // chunk offsets: a scan of the E chunk totals over the lanes
         int tA = lane < E ? sm.ld[lane].A : 0, tR = lane < E ? sm.ld[lane].PR : 0;
         long long tX = lane < E ? sm.ld[lane].PRA : 0;
@@ -811,8 +840,53 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                                (long long)jc * (np + 1))
                          : -CH_KV_MAX;
         }
-        hot_group_sync<NWG>();  // sm.ld / sm.ls are read
+        group_sync();  // sm.ld / sm.ls are read
     };
+    // (staged: from shared memory)
+    auto put_staged = [&](const Hot<EPL>& H, const ChOwn& own) CH_INLINE {
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) {
+            const int x = elem(e);
+            if (e * NWG * 32 > own.n) break;  // uniform
+            sm.str[x] = H.r[e];
+            sm.sta[x] = H.a[e] | ((H.pend >> e) & 1u ? (int)0x80000000 : 0);
+            sm.stS[x] = H.Sb[e];
+            sm.stk[x] = H.kv[e];
+            sm.stK[x] = H.SK[e];
+            sm.stb[x] = get_hb(H, e);
+            sm.sty[x] = get_hy(H, e);
+            sm.std_[x] = get_hd(H, e);
+        }
+        if (q == 0 && lane == 0) sm.sto = own;
+    };
+    auto get_staged = [&](Hot<EPL>& H, ChOwn& own) CH_INLINE {
+        own = sm.sto;
+        H.n = own.n;
+        H.M = own.M;
+        H.s = own.s;
+        H.inv_s = own.inv_s;
+        H.sumP = own.sumP;
+        H.pend = 0;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) {
+            const int x = elem(e);
+            H.num[e] = H.sg[e] = f_inf();
+            H.r[e] = H.a[e] = H.Sb[e] = 0;
+            H.SK[e] = 0;
+            H.kv[e] = -CH_KV_MAX;
+            set_consts(H, e, f_inf(), 0.0f, 0.0f, 0);
+            if (e * NWG * 32 > own.n) continue;  // uniform
+            const int a = sm.sta[x];
+            H.r[e] = sm.str[x];
+            H.a[e] = a & 0x7fffffff;
+            H.pend |= (unsigned)(a < 0) << e;
+            H.Sb[e] = sm.stS[x];
+            H.kv[e] = sm.stk[x];
+            H.SK[e] = sm.stK[x];
+            set_consts(H, e, sm.stb[x], sm.sty[x], sm.std_[x], sat((long long)hc * H.r[e]));
+        }
+    };
+
     // whether this warp's requests admit the candidate
     auto test = [&](const Hot<EPL>& H, const CandRec& cq, int a_in, auto ea) CH_INLINE {
         constexpr int EA = decltype(ea)::value;
@@ -1225,23 +1299,26 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                                        SMx == -CH_KV_MAX ? 0 : SMx, pmA, pmAp, smS, smSp);
             put_row(row, rr, next, o);
         }
-        if (q == NWG - 1 && lane == 31) {  // row 0 and the worker's own entries
+        // row 0, the worker's record, and its key: a warp each
+        if (q == NWG - 1 && lane == 31) {
             const int r0 = (int)(sm.key[0] >> 10);
             const RowVals o = make_row(P, H.inv_s, H.M, sumP, 0, r0, n, tot_a, 0, 0, LL_NONE, SM0,
                                        f_inf(), f_inf(), smS0, smSp0);
             put_row(0, 0, r0, o);
+            C.R[w] = R;
+            mR[m] = R;
+        } else if (q == 0 && lane == 0) {
             float4 wr = worker_record(P, H.inv_s, own.off, (float)own.sumP, own.wpmax, own.npend);
             wr.w = rank_bits;
-            const unsigned long long kq = norm_key(P, n, own.sumIn, own.sumPred);
-            C.R[w] = R;
             C.wrec[w] = wr;
+            mwrec[m] = wr;
+        } else if (q == 1 && lane == 0) {
+            const unsigned long long kq = hot_key(n, own.sumIn, own.sumPred);
             C.key[w] = kq;
+            mkey[m] = kq;
             if (P.approx)
                 C.wapx[w] = approx_bounds(P, C.scaled[w], own.dmin, n, own.sumP, own.sumIn,
                                           own.sumPred);
-            mR[m] = R;
-            mwrec[m] = wr;
-            mkey[m] = kq;
             sm.left_n = n;
         }
         hot_group_sync<NWG>();  // the scratch is free
@@ -1292,8 +1369,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 });
                 won = false;
                 alt_end = min(c + CH_SCAN, n_cand);
+                votes_sync();  // the sums are in: CH_TERMS forms candidate c's terms
                 cta_sync();
-                votes_sync();  // CH_TERMS has formed candidate c's terms
             }
             int k = c, d = CH_NOBODY;
             while (k < alt_end && d != CH_END)
@@ -1325,7 +1402,12 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 const float4 rcv = sm.rc[b];
                 if (sm.hw[v] != NONE) leave(H);
                 ChOwn own;
-                load(H, own, w);
+                if constexpr (Cfg::STAGE) {
+                    staged_wait<NWG>();
+                    get_staged(H, own);
+                } else {
+                    load(H, own, w);
+                }
                 const int n0 = H.n;
                 with_elems(n0 + 1, [&](auto ea) CH_INLINE { partial_sums(H, rw.y, c & 1, ea); });
                 hot_group_sync<NWG>();
@@ -1401,8 +1483,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 rerank();
                 prev = CH_NOBODY;
                 alt_end = min(c + CH_SCAN, n_cand);
-                cta_sync();
                 votes_sync();
+                cta_sync();
             }
             int code = CH_DONE, k = c;
             for (; k < alt_end; ++k) {
@@ -1545,10 +1627,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         for (int rp = 0; c < n_cand; rp ^= 1) {
             if (alt_end <= c) {
                 alt_end = min(c + CH_SCAN, n_cand);
-                cta_sync();
-                terms(o, c, false, false);
-                __syncwarp();
                 votes_sync();
+                terms(o, c, false, false);
+                cta_sync();
                 owed = false;
             }
             for (int k = c; k < alt_end; ++k) {
@@ -1626,10 +1707,18 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 break;
             }
             if (f & CH_UNMOD) mcount++;
-            // while the hot warps write the leaving worker's table and load w:
-            // w's requests towards L1, and the next candidates looked at among
-            // the workers other than the leaving one
-            {
+            // while the hot warps write the leaving worker's table: worker w is
+            // staged (or its requests fetched into L1), and the next candidates
+            // are looked at among the workers other than the leaving one
+            if constexpr (Cfg::STAGE) {
+                if (warp < CH_LOOK0 + NWG) {
+                    Hot<EPL> H;
+                    ChOwn own;
+                    load(H, own, w);
+                    put_staged(H, own);
+                    staged_arrive<NWG>();
+                }
+            } else {
                 const int nw = C.n[w];
                 const long long base = (long long)w * cap;
                 for (int x = 32 * ((warp - CH_LOOK0) * 32 + lane); x < nw; x += 32 * 32 * CH_SCAN) {
