@@ -201,7 +201,8 @@ int aladdin_score(aladdin_cluster* cl, int32_t n_cand, const int32_t* in, const 
  * validated and sorted on a second stream while the cluster's stream packs
  * the state and builds the tables; the two join before the scoring kernel,
  * and the call stays ordered on the cluster's stream like the two calls.
- * Otherwise it runs the two calls in sequence. */
+ * Otherwise, and where a call is small enough to be scored in one launch, it
+ * runs the two calls in sequence. */
 int aladdin_cluster_load_score(aladdin_cluster* cl, const int32_t* req_off, const int32_t* in,
                                const int32_t* gen, const int32_t* pred, const float* tdec_ms,
                                int32_t n_cand, const int32_t* cand_in, const int32_t* cand_pred,
@@ -350,13 +351,12 @@ int aladdin_cluster_status(aladdin_cluster* cl);
 int aladdin_cluster_test_waits(aladdin_cluster* cl, int64_t grid_polls, int64_t mbar_polls,
                                int32_t run_out);
 
-/* Test hook of the incremental placement round; the paper has no
- * counterpart. A best-fit round first scores every candidate against the
- * round-start state, then re-evaluates only the workers it modifies, holding
- * them in a bounded number of shared-memory slots; when they run out, the
- * round continues with the sliced round from the current state, and very
- * large rounds are split into chunks of candidates, each a fresh incremental
- * round. max_slots > 0 caps the slots and chunk > 0 the candidates per chunk,
+/* Test hook of the placement chain; the paper has no counterpart. A best-fit
+ * round evaluates every candidate against the round-start state and
+ * re-evaluates only the workers it modifies, holding them in a bounded number
+ * of shared-memory slots; when they run out, the round continues with the
+ * sliced round from the current state, and very large rounds are split into
+ * chunks of candidates, each a fresh chain. max_slots > 0 caps the slots and chunk > 0 the candidates per chunk,
  * so that tests reach both paths on small clusters (0: the defaults). The
  * placements do not depend on either. ALADDIN_ERR_ARG for negative values. */
 int aladdin_cluster_test_round(aladdin_cluster* cl, int32_t max_slots, int32_t chunk);

@@ -75,9 +75,9 @@ struct DevParams {
                                 // round's exchange waits for one arrival more than its
                                 // CTAs make; the scoring kernel withholds its first copy)
     int32_t round_slots_max;    // test hook (0: off): at most this many modified-worker
-                                // slots in the incremental round
+                                // slots in the placement chain
     int32_t round_chunk;        // test hook (0: off): at most this many candidates per
-                                // chunk of the incremental round
+                                // chunk of the placement chain
 };
 
 // Relative slack of a realized latency over its SLO before the execution step
@@ -450,13 +450,13 @@ struct BuildSmem {
 // Barrier of the NW warps building one table (NW consecutive warps of the
 // CTA when NW > 1; a named barrier, 1 unless the caller runs two builds side
 // by side, so that the other warps may run on).
-template <int NW, int BAR = 1>
+template <int NW>
 __device__ __forceinline__ void group_sync()
 {
     if constexpr (NW == 1) {
         __syncwarp();
     } else {
-        asm volatile("bar.sync %0, %1;" ::"n"(BAR), "r"(NW * 32) : "memory");
+        asm volatile("bar.sync %0, %1;" ::"n"(1), "r"(NW * 32) : "memory");
     }
 }
 
@@ -690,36 +690,34 @@ __device__ __forceinline__ void store_row(const ClusterDev& C, long long rowid, 
 // Shared-memory copies of one worker's breakpoints, record and key, kept by
 // the sliced placement round (pointers to this worker's entries).
 struct SliceCache {
-    unsigned short* rho;  // sample i: rho_{q+1} - 1 of row q = ((i + 1) << shift) - 1 < R
-    int rc;               // samples held
-    int shift;            // every (1 << shift)-th row is sampled
+    unsigned short* rho;  // entry q: rho_{q+1} - 1 of row q < R
+    int rc;               // entries held
     int* R;
     float4* wrec;
     unsigned long long* key;
 };
 
 // Build worker w's table (rows 0..R), its record and its capacity_norm key.
-// Called by all lanes of NW warps (warps W0..W0+NW-1 of the CTA when NW > 1,
-// synchronised by named barrier BAR); element x = (q EW + e) 32 + lane of
+// Called by all lanes of NW warps (the first NW of the CTA when NW > 1,
+// synchronised by named barrier 1); element x = (q EW + e) 32 + lane of
 // the group's warp q, so 32 EW NW slots are covered. Requests are loaded from
 // the slot arrays; an invalid request (in < 0, gen outside [0, pred), in +
 // pred > K) makes the worker infeasible for every candidate and sets err bit 1.
 // With `cache`, the worker's shared-memory copies are refreshed as well. With a
 // valid `cand`, the candidate is evaluated against the new table by the lane
 // that holds its row, and every lane returns its flags (else 0). INSERT: the
-// last request (1) or the last `ins` requests (2) were appended since the
-// build that left its sorted keys in skey, and are inserted into that order
-// instead of sorting afresh.
-template <int EW, int NW = 1, int INSERT = 0, int BAR = 1, int W0 = 0>
+// last request was appended since the build that left its sorted keys in skey,
+// and is inserted into that order instead of sorting afresh.
+template <int EW, int NW = 1, bool INSERT = false>
 __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
                                 BuildSmem<EW, NW>& sm, const SliceCache* cache = nullptr,
-                                const CandRec* cand = nullptr, int ins = 1)
+                                const CandRec* cand = nullptr)
 {
     static_assert(!INSERT || NW > 1, "the insertion path is for cooperative builds");
     constexpr int E = EW;
     constexpr int RUN = 32 * EW;  // elements per warp
     const int lane = threadIdx.x & 31;
-    const int q = NW > 1 ? (int)(threadIdx.x >> 5) - W0 : 0;
+    const int q = NW > 1 ? (int)(threadIdx.x >> 5) : 0;
     const int x0 = q * RUN;
     const long long base = (long long)w * C.cap;
     const long long rowbase = (long long)w * C.rows;
@@ -738,8 +736,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     double l_wt[EL];
     unsigned l_sk[INSERT ? E : 1];
     if constexpr (INSERT) {
-        // The previous build's sorted keys (all requests but the last `ins`,
-        // which were appended since).
+        // The previous build's sorted keys (all requests but the last).
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = x0 + e * 32 + lane;
@@ -827,7 +824,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             sm.pi[1][q] = bad;
         }
     }
-    group_sync<NW, BAR>();
+    group_sync<NW>();
     if constexpr (NW > 1) {
         sumP = combine_warps<NW>(sm.pll[0], OpAdd<long long>(), 0LL);
         sumIn = combine_warps<NW>(sm.pll[1], OpAdd<long long>(), 0LL);
@@ -853,7 +850,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
         for (int d = 16; d > 0; d >>= 1) dmin = fmin(dmin, __shfl_xor_sync(FULL, dmin, d));
         if constexpr (NW > 1) {
             if (lane == 0) sm.pdm[q] = dmin;
-            group_sync<NW, BAR>();
+            group_sync<NW>();
             dmin = combine_warps<NW>(sm.pdm, OpMin<double>(), dmin);
         }
         wa = approx_bounds(P, C.scaled[w], dmin, n, sumP, sumIn, sumPred);
@@ -872,7 +869,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     // keys below it (keys of valid requests are distinct); larger ones sort
     // each warp's run and merge the runs.
     constexpr bool COUNT_RANK = NW > 1 && N <= 256 && !INSERT;
-    if constexpr (INSERT == 1) {
+    if constexpr (INSERT) {
         // Insert the appended request's key into the previous sorted order: it
         // lands after the keys below it, the others move up by one.
         const int n0 = n - 1;
@@ -882,7 +879,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             if (x < n0) sm.runs[x] = l_sk[e];
             if (x == n0) sm.newk = key[e];
         }
-        group_sync<NW, BAR>();
+        group_sync<NW>();
         const unsigned nk = sm.newk;
         int lo;  // old keys below nk
         if constexpr (E == 1) {
@@ -892,7 +889,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n"
                          " bar.red.popc.u32 %0, %3, %1, p;\n}"
                          : "=r"(cnt)
-                         : "r"(NW * 32), "r"(below), "n"(BAR)
+                         : "r"(NW * 32), "r"(below), "n"(1)
                          : "memory");
             lo = (int)cnt;
         } else {
@@ -911,51 +908,8 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
         }
         if (q == 0 && lane == 0) sm.sorted[lo] = nk;
     }
-    if constexpr (INSERT == 2) {
-        // Several appended requests: every key moves up by the appended keys
-        // below it, counted one by one; an appended key also by the old ones,
-        // found by a search.
-        const int n0 = n - ins;
-        unsigned* newk = reinterpret_cast<unsigned*>(sm.kvrho);  // not in use yet
-        const int pad = (ins + 3) & ~3;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int x = x0 + e * 32 + lane;
-            if (x < n0) sm.runs[x] = l_sk[e];
-            else if (x < n0 + pad) newk[x - n0] = x < n ? key[e] : 0xffffffffu;
-        }
-        for (int j = ins + q * 32 + lane; j < pad; j += 32 * NW) newk[j] = 0xffffffffu;
-        group_sync<NW, BAR>();
-        unsigned mine[E];
-        int at[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int x = x0 + e * 32 + lane;
-            mine[e] = x < n0 ? l_sk[e] : key[e];
-            at[e] = x;
-            if (x >= n0 && x < n) {
-                int lo = 0, hi = n0;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (sm.runs[mid] < mine[e]) lo = mid + 1;
-                    else hi = mid;
-                }
-                at[e] = lo;
-            }
-        }
-        const uint4* new4 = reinterpret_cast<const uint4*>(newk);
-        for (int k = 0; k < pad / 4; ++k) {
-            const uint4 v = new4[k];
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                at[e] += (v.x < mine[e]) + (v.y < mine[e]) + (v.z < mine[e]) + (v.w < mine[e]);
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-            if (x0 + e * 32 + lane < n) sm.sorted[at[e]] = mine[e];
-    }
-    if constexpr (INSERT != 0) {
-        group_sync<NW, BAR>();
+    if constexpr (INSERT) {
+        group_sync<NW>();
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = x0 + e * 32 + lane;
@@ -965,7 +919,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     if constexpr (COUNT_RANK) {
 #pragma unroll
         for (int e = 0; e < E; ++e) sm.runs[x0 + e * 32 + lane] = key[e];
-        group_sync<NW, BAR>();
+        group_sync<NW>();
         int rank[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) rank[e] = 0;
@@ -980,7 +934,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
 #pragma unroll
         for (int e = 0; e < E; ++e)
             if (x0 + e * 32 + lane < n) sm.sorted[rank[e]] = key[e];
-        group_sync<NW, BAR>();
+        group_sync<NW>();
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = x0 + e * 32 + lane;
@@ -1022,7 +976,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
         // earlier runs first).
 #pragma unroll
         for (int e = 0; e < E; ++e) sm.runs[x0 + e * 32 + lane] = key[e];
-        group_sync<NW, BAR>();
+        group_sync<NW>();
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             // In every other run, the count of keys before this one: a
@@ -1047,7 +1001,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
                 if (q2 != q) rank += cnt[q2];
             sm.sorted[rank] = key[e];
         }
-        group_sync<NW, BAR>();
+        group_sync<NW>();
 #pragma unroll
         for (int e = 0; e < E; ++e) key[e] = sm.sorted[x0 + e * 32 + lane];
     }
@@ -1130,7 +1084,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             sm.pll[4][q] = s_ra.total;
             sm.pi[4][q] = s_a.total;
         }
-        group_sync<NW, BAR>();
+        group_sync<NW>();
         add_carry_prefix<NW>(s_row, sm.pi[2], q);
         add_carry_prefix<NW>(s_r, sm.pi[3], q);
         add_carry_prefix<NW>(s_ra, sm.pll[4], q);
@@ -1157,7 +1111,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             sm.Tp[rowid[e]] = decode_time(P, s, (float)rr, (float)Sb, (float)SK);
         }
     }
-    group_sync<NW, BAR>();
+    group_sync<NW>();
 
     // Per-request bounds and slacks.
     const float stallk = P.k1 * (float)sumP + P.c1;
@@ -1209,7 +1163,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             sm.pf[4][q] = s_smSp.total;
             sm.pll[1][q] = s_SM.total;
         }
-        group_sync<NW, BAR>();
+        group_sync<NW>();
         add_carry_prefix<NW>(s_pmA, sm.pf[1], q);
         add_carry_prefix<NW>(s_pmAp, sm.pf[2], q);
         add_carry_prefix<NW>(s_PM, sm.pll[0], q);
@@ -1243,11 +1197,8 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
                 const RowVals o = make_row(P, inv_s, M, sumP, r[e], nxt, np, A, pre_r[e], pre_ra[e],
                                            PMx[e], SM, pmA[e], pmAp[e], smS[e], smSp[e]);
                 store_row(C, rowbase + rowid[e], o, P.want_aux != 0);
-                if (cache) {
-                    const int q1 = rowid[e] + 1, sh = cache->shift, i = (q1 >> sh) - 1;
-                    if (rowid[e] < R && i >= 0 && i < cache->rc && (q1 & ((1 << sh) - 1)) == 0)
-                        cache->rho[i] = (unsigned short)(nxt - 1);
-                }
+                if (cache && rowid[e] < R && rowid[e] < cache->rc)
+                    cache->rho[rowid[e]] = (unsigned short)(nxt - 1);
                 if (want && r[e] <= rc && rc < nxt) {
                     float m;
                     cf = eval_pair_mode(P.approx, o.v0, o.v1, o.ext, wr, wa, *cand, m);
@@ -1279,8 +1230,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
         if (P.approx) C.wapx[w] = wa;
         C.key[w] = kq;
         if (cache) {
-            if (!bad && n > 0 && R > 0 && cache->shift == 0)
-                cache->rho[0] = (unsigned short)(r0 - 1);
+            if (!bad && n > 0 && R > 0) cache->rho[0] = (unsigned short)(r0 - 1);
             *cache->R = bad ? 0 : R;
             *cache->wrec = wr;
             *cache->key = kq;
@@ -1288,7 +1238,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     }
     if constexpr (NW > 1) {
         if (mine) sm.cflag = cf;  // exactly one lane of the group holds the row
-        group_sync<NW, BAR>();
+        group_sync<NW>();
         return want ? sm.cflag : 0u;
     } else {
         __syncwarp();
@@ -1303,24 +1253,24 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
 // elements, not 1,024). smem holds a BuildSmem<EWMAX, NW>; the smaller
 // variants use a prefix of it. n is the worker's current count (uniform over
 // the NW warps).
-template <int EWMAX, int NW, int INSERT = 0, int BAR = 1, int W0 = 0>
+template <int EWMAX, int NW, bool INSERT = false>
 __device__ __forceinline__ unsigned build_table_fit(const DevParams& P, const ClusterDev& C, int w,
                                                     int n, unsigned char* smem,
                                                     const SliceCache* cache = nullptr,
-                                                    const CandRec* cand = nullptr, int ins = 1)
+                                                    const CandRec* cand = nullptr)
 {
     if constexpr (EWMAX >= 4) {
         if (n > 64 * NW)  // more than the EW = 2 variant covers
-            return build_table<4, NW, INSERT, BAR, W0>(
-                P, C, w, *reinterpret_cast<BuildSmem<4, NW>*>(smem), cache, cand, ins);
+            return build_table<4, NW, INSERT>(
+                P, C, w, *reinterpret_cast<BuildSmem<4, NW>*>(smem), cache, cand);
     }
     if constexpr (EWMAX >= 2) {
         if (n > 32 * NW)
-            return build_table<2, NW, INSERT, BAR, W0>(
-                P, C, w, *reinterpret_cast<BuildSmem<2, NW>*>(smem), cache, cand, ins);
+            return build_table<2, NW, INSERT>(
+                P, C, w, *reinterpret_cast<BuildSmem<2, NW>*>(smem), cache, cand);
     }
-    return build_table<1, NW, INSERT, BAR, W0>(
-        P, C, w, *reinterpret_cast<BuildSmem<1, NW>*>(smem), cache, cand, ins);
+    return build_table<1, NW, INSERT>(
+        P, C, w, *reinterpret_cast<BuildSmem<1, NW>*>(smem), cache, cand);
 }
 
 }  // namespace aladdin

@@ -105,7 +105,7 @@ struct RoundIO {
     // simulations that run side by side with others
     int single_cta;
     // direct mode: device pointer to the first candidate still to place (the
-    // ones before it were placed by the incremental round), or nullptr (0)
+    // ones before it were placed by the chain), or nullptr (0)
     const int* c_first;
     // direct mode: some worker holds requests placed earlier in the open round
     int round_open;

@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(R2_THREADS, 1) k_round2(R2Args A)
 {
     constexpr int NW = R2Split<E>::NW, EW = R2Split<E>::EW;
     // the winner's previous sorted order is current: insert its new key
-    constexpr int NW_INSERT = NW > 1 ? 1 : 0;
+    constexpr bool NW_INSERT = NW > 1;
     extern __shared__ __align__(16) unsigned char smraw[];
     R2Smem<E>& sm = *reinterpret_cast<R2Smem<E>*>(smraw);
     const int cap = A.C.cap;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(R2_THREADS, 1) k_round2(R2Args A)
     const ClusterDev& C = A.C;
     const RoundIO& io = A.io;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // direct mode after the incremental round: the candidates before c_begin
+    // direct mode after the placement chain: the candidates before c_begin
     // are placed already (every CTA reads the same value)
     const int c_begin = (!io.sim && io.c_first) ? *io.c_first : 0;
     if (!io.sim && c_begin >= io.n_cand) return;
@@ -304,12 +304,12 @@ __global__ void __launch_bounds__(R2_THREADS, 1) k_round2(R2Args A)
     // of the CTA takes the same branch (and the same barrier).
     auto rebuild = [&](int w, bool small, const CandRec* cand) -> unsigned {
         const int lw = w - w_lo;
-        SliceCache sc{rho + (long long)lw * rs, rc, 0, &R_s[lw], &wrec_s[lw], &key_s[lw]};
+        SliceCache sc{rho + (long long)lw * rs, rc, &R_s[lw], &wrec_s[lw], &key_s[lw]};
         append(w);
         if constexpr (NW > 4) {
             if (small) {
                 group_sync<4>();
-                return build_table_fit<1, 4, 1>(P, C, w, n_s[lw],
+                return build_table_fit<1, 4, true>(P, C, w, n_s[lw],
                                                    reinterpret_cast<unsigned char*>(&sm.build),
                                                    &sc, cand);
             }

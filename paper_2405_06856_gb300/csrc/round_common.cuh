@@ -1,5 +1,5 @@
 // Device helpers of the two best-fit round kernels (the sliced round k_round2
-// and the incremental round k_round_inc): the rebuild group's split, the
+// and the placement chain k_round_chain): the rebuild group's split, the
 // shared-memory breakpoint search and the (key, lowest index) reductions.
 #pragma once
 
