@@ -1,0 +1,159 @@
+"""The placement chain (k_round_chain) at the sizes where it changes shape:
+tables of each size class whose workers cross the register steps, rounds with
+and without the flag matrix, groups, every option that changes a bound, and
+simulations; against the oracle, through the C ABI."""
+import numpy as np
+import pytest
+
+from parity import NEAR, compare_pairs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def A():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.init()
+    from paper_2405_06856_gb300 import build
+    build.build()
+    from paper_2405_06856_gb300 import aladdin
+    return aladdin
+
+
+LOOSE = dict(T_pre=1e5, T_dec=400.0)
+REFUSED = -2
+HIST = dict(lo_ms=8.0, hi_ms=20.0)
+
+# W, slots, requests a worker at first (at most), KV, candidates, parameters.
+# A hot worker's lanes hold one request more at every 128 (more than four a
+# lane: 512 slots and up step at 256, 384, 512), so the first rows fill
+# workers across those counts; the others are the dispatch's edges (192
+# workers, 64 candidates) and the options.
+ROUNDS = {
+    "slots32": (40, 32, 8, 9000, 300, dict(T_pre=200.0)),
+    "slots128": (12, 128, 60, 50000, 500, LOOSE),
+    "slots256-over-128": (6, 256, 120, 105000, 500, LOOSE),
+    "slots512-over-128-256-384": (4, 512, 250, 240000, 900, LOOSE),
+    "slots1024-over-256-384-512": (3, 1024, 380, 420000, 1500, LOOSE),
+    "slots1024-fill": (8, 1024, 10, 60000, 900, dict(T_pre=150.0)),
+    "table-191": (191, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
+    "flags-192": (192, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
+    "table-63": (700, 128, 30, 40000, 63, dict(T_pre=300.0, T_dec=20.0)),
+    "flags-64": (700, 128, 30, 40000, 64, dict(T_pre=300.0, T_dec=20.0)),
+    "flags-many-words": (1100, 64, 20, 20000, 600, dict(T_pre=200.0, T_dec=11.0)),
+    "one-candidate": (20, 128, 30, 40000, 1, {}),
+    "one-worker-fills": (1, 256, 30, 30000, 150, LOOSE),
+    "groups3": (100, 256, 40, 60000, 400, dict(groups=3, T_dec=30.0)),
+    "groups7-ragged-fill": (17, 512, 40, 30000, 600, dict(groups=7, T_dec=30.0)),
+    "gamma-h-j": (60, 256, 40, 90000, 300, dict(gamma=0.3, h=2, j=3, T_pre=400.0, T_dec=24.0)),
+    "theta-history": (60, 256, 40, 90000, 300, dict(theta=0.85, T_pre=400.0, T_dec=26.0, hist=1)),
+    "approx-history": (60, 256, 40, 90000, 300,
+                       dict(mode=1, theta=0.9, T_pre=200.0, T_dec=26.0, hist=1)),
+    "approx-flags": (260, 256, 40, 90000, 300,
+                     dict(mode=1, theta=0.9, T_pre=200.0, T_dec=26.0, hist=1)),
+    "decode": (60, 256, 40, 90000, 300, dict(phase=1, T_dec=26.0, hist=1)),
+}
+
+
+def workload(synth, name):
+    W, cap, per, kv, n, p = ROUNDS[name]
+    p = dict(p)
+    hist = p.pop("hist", 0)
+    seed = 700 + list(ROUNDS).index(name)
+    wl = synth.make_cluster("chain", seed, W, per, kv, n, per_worker_random=True, b_cap=cap,
+                            gpus_cycle=(1, 2) if "history" in name else (1,), params=p)
+    wl.cand_pred[max(n // 2, 1)::17] = 0  # refused candidates inside the runs
+    return wl, synth.decode_history(wl, HIST["lo_ms"], HIST["hi_ms"], seed) if hist else None
+
+
+def oracle_cluster(orc, wl, tdec):
+    return orc.Cluster.from_workload(wl, tdec=None if tdec is None else tdec.astype(np.float64))
+
+
+def oracle_round(oc, wl, lo, hi):
+    """Candidates [lo, hi); the refused ones are not handed to the oracle."""
+    c = np.arange(lo, hi)
+    ok = wl.cand_pred[lo:hi] > 0
+    out = np.full(hi - lo, REFUSED, np.int32)
+    out[ok] = oc.place_round(wl.cand_in[c[ok]], wl.cand_pred[c[ok]], wl.cand_wait[c[ok]], crid=c[ok])
+    return out
+
+
+@pytest.mark.parametrize("name", list(ROUNDS))
+def test_chain_places_like_the_oracle(A, orc, synth, name):
+    """Two calls of one open round, and scoring against the tables that the
+    chain left. A pair whose slack is within the fp32 bar of zero may go
+    either way; the first divergence, if any, must be such a pair of the
+    candidate's group."""
+    wl, tdec = workload(synth, name)
+    n, G = wl.n_cand, wl.params.get("groups", 1)
+    oc = oracle_cluster(orc, wl, tdec)
+    cut = n - n // 3
+    with A.Cluster.from_workload(wl, tdec_ms=tdec) as cl:
+        pl, rl = [], []
+        for lo, hi in ((0, cut), (cut, n)):
+            if lo == hi:
+                continue
+            q = (wl.cand_in[lo:hi], wl.cand_pred[lo:hi], wl.cand_wait[lo:hi])
+            pl.append(cl.place_round(*q))
+            rl.append(oracle_round(oc, wl, lo, hi))
+        assert cl.status() == A.OK
+        pl, rl = np.concatenate(pl), np.concatenate(rl)
+        mis = np.flatnonzero(pl != rl)
+        if len(mis):
+            c = int(mis[0])
+            o2 = oracle_cluster(orc, wl, tdec)
+            oracle_round(o2, wl, 0, c)
+            r = o2.score(wl.cand_in[c:c + 1], wl.cand_pred[c:c + 1], wl.cand_wait[c:c + 1])
+            ws = np.arange(wl.n_workers)
+            assert (r["near"][0, ws % G == c % G] <= NEAR).any(), (c, pl[c], rl[c])
+            return
+        assert (pl >= 0).any()
+        k = min(n, 40)
+        ok = wl.cand_pred[:k] > 0
+        q = (wl.cand_in[:k][ok], wl.cand_pred[:k][ok], wl.cand_wait[:k][ok])
+        g = cl.score(*q, detail=True)
+        compare_pairs(oc.score(*q), g["flags"], g["margin"], q[0], g["kvpeak"], g["tcand"], name)
+        counts = cl.state()[0]
+        assert np.array_equal(counts, oc.n)
+
+
+@pytest.mark.parametrize("N,cap,kv,rate,extra", [
+    (7, 64, 16000, 30.0, {}),
+    (6, 128, 40000, 60.0, dict(gamma=0.3)),
+    (5, 512, 120000, 120.0, dict(T_dec=40.0)),
+    (3, 1024, 300000, 160.0, dict(T_dec=80.0)),
+    (9, 256, 40000, 60.0, dict(rebalance=1, theta=0.9)),
+    (2047, 32, 6000, 3000.0, dict(T_dec=14.0)),
+    (2049, 32, 6000, 3000.0, dict(T_dec=14.0)),   # more workers than the chain ranks by itself
+])
+def test_chain_simulates_like_the_oracle(A, orc, synth, N, cap, kv, rate, extra):
+    tr = synth.diurnal_trace(40 + N, 700, rate, rate / 4)
+    p = dict(synth.BASE_PARAMS, **extra)
+    ref = orc.simulate(p, N, cap, kv, 1.0, tr, 100.0, stop_at_fail=False, drain=True)
+    out = np.zeros(A.SIMULATE_OUT)
+    A.aladdin_simulate(A.make_params(p, cap), A.make_cfgs([1], [kv], [1.0])[0], N,
+                       A.trace_of(tr), 100.0, 0, 1, out)
+    assert int(out[0]) == ref["failed"] and int(out[1]) == ref["placed"], (out, ref)
+    assert int(out[2]) == ref["heartbeats"] and int(out[5]) == ref["violations"], (out, ref)
+    assert out[3] == pytest.approx(ref["max_ttft"], rel=1e-12)
+    assert out[4] == pytest.approx(ref["max_atgt"], rel=1e-12)
+    assert int(out[8]) == ref["moved"]
+
+
+def test_exact_predictions_equal_real_lengths(A, synth):
+    """The execution step has a branch of its own where predictions are exact;
+    a trace that states the same lengths as the real ones takes the general
+    branch and must end with the same numbers, bit for bit."""
+    tr = synth.diurnal_trace(77, 1500, 80.0, 20.0)
+    p = dict(synth.BASE_PARAMS, T_dec=30.0)
+    outs = []
+    for real in (None, np.asarray(tr.req_pred)):
+        t = synth.Trace(tr.t_arr, tr.req_in, tr.req_pred, real, None)
+        out = np.zeros(A.SIMULATE_OUT)
+        A.aladdin_simulate(A.make_params(p, 256), A.make_cfgs([1], [40000], [1.0])[0], 6,
+                           A.trace_of(t), 100.0, 0, 1, out)
+        outs.append(out)
+    assert outs[0][1] > 0 and outs[0].tobytes() == outs[1].tobytes()
