@@ -447,16 +447,15 @@ struct BuildSmem {
     uint8_t pend[N];
 };
 
-// Barrier of the NW warps building one table (NW consecutive warps of the
-// CTA when NW > 1; a named barrier, 1 unless the caller runs two builds side
-// by side, so that the other warps may run on).
+// Barrier of the NW warps building one table (the first NW warps of the CTA
+// when NW > 1; a named barrier, so that the other warps may run on).
 template <int NW>
 __device__ __forceinline__ void group_sync()
 {
     if constexpr (NW == 1) {
         __syncwarp();
     } else {
-        asm volatile("bar.sync %0, %1;" ::"n"(1), "r"(NW * 32) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"r"(NW * 32) : "memory");
     }
 }
 

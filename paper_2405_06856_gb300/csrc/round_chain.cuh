@@ -187,7 +187,7 @@ struct ChSmem {
     int code[2], next[2];            // [run parity]
     int miss_w, miss_f, victim;
     int left_n;                      // requests of the worker that left last
-    int abort;
+    int abort, never;                // a run has ended; always 0
     int cnt[CH_WARPS + 1];
     int lq[CH_SCAN][64];             // look-ahead: slots to evaluate
 };
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         for (int k = lane; k < rec_end; k += 32) fetch(k);
     if (A.F && warp >= CH_LOOK0)
         for (int k = warp - CH_LOOK0; k < rec_end; k += CH_SCAN) fetch_row(k);
-    if (tid == 0) sm.abort = 0;
+    if (tid == 0) sm.abort = sm.never = 0;
     __syncthreads();
 
     int mcount = 0;  // modified workers (every thread tracks the same value)
@@ -476,7 +476,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
 
     // A look-ahead warp: candidate k's best choice among the workers that are
     // not hot.
-    auto look = [&](int k) CH_INLINE {
+    auto look = [&](int k, const int* stop) CH_INLINE {
+        auto stopped = [&]() { return __any_sync(FULL, *(const volatile int*)stop) != 0; };
         const int b = k & (CH_RING - 1);
         const CandRec cq = sm.rec[b];
         unsigned long long bk = 0ull;
@@ -507,6 +508,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 }
             } else {
                 for (int base = 0; base < W; base += 32) {
+                    if (stopped()) return;
                     const int pos = base + lane;
                     bool ok = false;
                     RankEnt e{0ull, 0, 0};
@@ -1674,7 +1676,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             if (alt_end <= c) {
                 alt_end = min(c + CH_SCAN, n_cand);
                 const int k = c + warp - CH_LOOK0;
-                if (!primed && k < alt_end) look(k);
+                if (!primed && k < alt_end) look(k, &sm.never);
                 primed = false;
                 cta_sync();
             }
@@ -1691,7 +1693,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             rec_end = rec_new;
             for (int k = alt_end + warp - CH_LOOK0; k < new_end; k += CH_SCAN) {
                 if (__any_sync(FULL, *(volatile int*)&sm.abort)) break;
-                look(k);
+                look(k, &sm.abort);
             }
             cta_sync();
             const int code = sm.code[rp];
@@ -1732,7 +1734,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             }
             c += 1;
             const int k = c + warp - CH_LOOK0;
-            if (k < n_cand) look(k);
+            if (k < n_cand) look(k, &sm.never);
             cta_sync();
             if (sm.hw[v] != NONE) {  // now the one that left
                 const int i = sm.hm[v], n = sm.left_n, b = k & (CH_RING - 1);
