@@ -66,7 +66,11 @@ constexpr int CH_TERMS = CH_HOT + 1;          // the warp that forms the workers
 constexpr int CH_LOOK0 = CH_HOT + 2;          // first warp looking ahead
 constexpr int CH_SCAN = CH_WARPS - CH_LOOK0;  // warps looking ahead
 constexpr int CH_RING = 64;                   // candidate records in shared memory
-constexpr int CH_AHEAD = 18;                  // candidates looked ahead at a time
+// Candidates looked ahead at a time: a miss makes looks useless, and looks slow
+// the links beside them. 30, 18 and 12 took a round of 256 workers 1.82, 1.67
+// and 1.68 ms, a simulation of 128 workers 25.2, 24.0 and 23.6 ms, eight groups
+// 0.96, 0.90 and 0.87 ms.
+constexpr int CH_AHEAD = 12;
 constexpr int CH_WIN = 1024;                  // rank positions kept in shared memory
 constexpr int CH_SORT_MAX = 2048;             // workers a trace-mode round ranks by itself
 constexpr int CH_MAX_SLOTS = 4096;            // modified workers held, at most
