@@ -7,9 +7,9 @@
 // a request to i: every other worker keeps its state, its table and its
 // capacity_norm. And most candidates go to a worker that took one of the last
 // few (best fit fills the fullest worker that still takes the request; two to
-// eight workers receive 90-98% of a round). So the chain keeps the last few
-// winners "hot": their requests sit in the registers of one to four warps
-// each, with the exact integer aggregates of the projection at each request's
+// eight workers receive 90-98% of a round). So the chain keeps two of the
+// last winners "hot": their requests sit in the registers of four warps each,
+// with the exact integer aggregates of the projection at each request's
 // last iteration (iterations and context tokens run until then, KV held at
 // it). For a hot worker
 //   * a candidate's test needs no table: each request tests the candidate's
@@ -20,21 +20,26 @@
 //   * an appended request changes each aggregate by a term of its own, so
 //     nothing is sorted or scanned: a link updates the aggregates, re-forms
 //     the bounds and tests the next candidate.
-// The other half of the CTA's warps look ahead: for each of the next
-// candidates they find its best choice among the workers that are not hot
-// (the first feasible worker the round has not modified, in the round-start
-// capacity_norm order, and the feasible modified worker of largest key). A
-// link then compares the hot workers with that one record. Only when the
-// record wins (a "miss") does a worker change places: its requests are loaded
-// and summed (its sorted keys are kept by every table build), the hot worker
-// used least recently leaves, its table formed from its aggregates (the same
-// values as a table build's, without its sorts and sums), and the look-ahead
-// starts anew.
+// Of the CTA's 16 warps eight hold the hot workers; one decides each link from
+// their votes and the look-ahead's record; one forms the hot workers' own terms
+// (KV at the candidate's end, TTFT, the candidate's own decode bound); six look
+// ahead: for each of the next candidates they find its best choice among the
+// workers that are not hot (the first feasible worker the round has not
+// modified, in the round-start capacity_norm order, and the feasible modified
+// worker of largest key). Only when that record wins (a "miss") does a worker
+// change places: the hot worker used least recently leaves, its table formed
+// from its aggregates (the same values as a table build's, without its sorts
+// and sums), while look-ahead warps load and sum the new worker's requests (its
+// sorted keys are kept by every table build; beyond 512 slots the hot warps do
+// that themselves afterwards) and look at the next candidates among the others.
 //
-// Bound: the link's latency, about 30 dependent steps of register arithmetic,
-// a vote, a barrier of the hot warps and a reduction. Rebuilding the winner's
-// table at every link instead took 2.4 us a candidate on 128-slot tables and
-// 6.4 us on 1,024-slot ones.
+// Bound: the link's latency, a chain of dependent register arithmetic, a vote,
+// two barriers and a reduction at 45% of the SM's issue slots. On tables of up
+// to 128, 512 and 1,024 slots a plain link takes 1,150, 1,300 and 1,790 cycles
+// and a miss 7,000, 11,000 and 28,000. Measured against rebuilding the winner's
+// table at every link: 2,048 candidates on 256 workers 5.3 -> 1.68 ms, 13,107 on
+// 16,384 workers (1,024 slots) 84 -> 18 ms, 31 groups on 4,096 workers 2.75 ->
+// 0.87 ms, a simulation of 128 workers 37.2 -> 23.6 ms.
 //
 // Where the round has a candidate x worker flag matrix (direct rounds of
 // larger fleets, scored by the scoring kernel against the round-start state in
@@ -68,8 +73,8 @@ constexpr int CH_SCAN = CH_WARPS - CH_LOOK0;  // warps looking ahead
 constexpr int CH_RING = 64;                   // candidate records in shared memory
 // Candidates looked ahead at a time: a miss makes looks useless, and looks slow
 // the links beside them. 30, 18 and 12 took a round of 256 workers 1.82, 1.67
-// and 1.68 ms, a simulation of 128 workers 25.2, 24.0 and 23.6 ms, eight groups
-// 0.96, 0.90 and 0.87 ms.
+// and 1.68 ms, a simulation of 128 workers 25.2, 24.0 and 23.6 ms, 31 groups on 4,096
+// workers 0.96, 0.90 and 0.87 ms.
 constexpr int CH_AHEAD = 12;
 constexpr int CH_WIN = 1024;                  // rank positions kept in shared memory
 constexpr int CH_SORT_MAX = 2048;             // workers a trace-mode round ranks by itself
@@ -86,10 +91,16 @@ constexpr int CH_HJ_MAX = 1 << 25;            // h and j likewise: one token wou
 // over NWG warps; KH hot workers.
 template <int E>
 struct ChCfg {
-    static constexpr int NWG = 4;
+    static constexpr int NWG = E >= 32 ? 8 : 4;
     static constexpr int EPL = E / NWG;
     static constexpr int KH = CH_HOT / NWG;
-    static constexpr bool STAGE = EPL <= 4;  // look-ahead warps load the next hot worker
+    // look-ahead warps that load the next hot worker, their elements a lane, and
+    // the requests that they hold
+    static constexpr int LN = 4, LE = EPL, LCAP = 32 * LN * LE;
+    static __device__ __forceinline__ bool staged(int n)
+    {
+        return NWG == LN || (n > 128 && n < LCAP);
+    }
 };
 
 // Round-start entry of a rank position: the worker there, its key and count.
@@ -181,7 +192,7 @@ struct ChSmem {
     float ebnd[32 * E], esg[32 * E];
     // a worker that becomes hot, formed by look-ahead warps while the hot ones
     // write the leaving worker's table (bit 31 of sta: placed in this round)
-    static constexpr int ST = Cfg::STAGE ? 32 * E : 1;
+    static constexpr int ST = Cfg::LCAP;
     int str[ST], sta[ST], stS[ST], stk[ST];
     long long stK[ST];
     float stb[ST], sty[ST], std_[ST];
@@ -233,12 +244,12 @@ __device__ __forceinline__ void stage_group_sync()
 template <int N>
 __device__ __forceinline__ void staged_arrive()
 {
-    asm volatile("bar.arrive 7, %0;" ::"r"(2 * N * 32) : "memory");
+    asm volatile("bar.arrive 7, %0;" ::"r"(N * 32) : "memory");
 }
 template <int N>
 __device__ __forceinline__ void staged_wait()
 {
-    asm volatile("bar.sync 7, %0;" ::"r"(2 * N * 32) : "memory");
+    asm volatile("bar.sync 7, %0;" ::"r"(N * 32) : "memory");
 }
 
 // A link's two barriers: votes and terms are in (hot warps, CH_DECIDE and
@@ -697,12 +708,16 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         }
         return t;
     };
-    // load worker w's requests into the registers of NWG warps
-    auto group_sync = [&]() CH_INLINE {
-        if constexpr (Cfg::STAGE) stage_group_sync<NWG>();
-        else hot_group_sync<NWG>();
-    };
-    auto load = [&](Hot<EPL>& H, ChOwn& own, int w) CH_INLINE {
+    // load worker w's requests into the registers of LN warps
+    auto load = [&](auto& H, ChOwn& own, int w, auto ln) CH_INLINE {
+        constexpr int LN = decltype(ln)::value, LE = EPL, LC = LE * LN;
+        constexpr bool HOT = LN == NWG && NWG > Cfg::LN;  // by the hot warps themselves
+        const int q = warp % LN;
+        auto elem = [&](int e) CH_INLINE { return (e * LN + q) * 32 + lane; };
+        auto group_sync = [&]() CH_INLINE {
+            if constexpr (HOT) hot_group_sync<LN>();
+            else stage_group_sync<LN>();
+        };
         const long long base = (long long)w * cap;
         const int n = C.n[w];
         H.n = n;
@@ -722,12 +737,12 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         // Sb, kv, SK first hold the inclusive prefix sums of r, a and
         // r a + r (r + 1) / 2 inside the chunk of 32
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) {
+        for (int e = 0; e < LE; ++e) {
             const int x = elem(e);
             H.r[e] = H.a[e] = H.Sb[e] = H.kv[e] = 0;
             H.SK[e] = 0;
             set_consts(H, e, f_inf(), 0.0f, 0.0f, 0);
-            if (e * NWG * 32 >= n) continue;
+            if (e * LN * 32 >= n) continue;
             float hb = f_inf(), hy = 0.0f, hd = 0.0f;
             if (x < n) {
                 const unsigned key = C.skey[base + x];
@@ -758,8 +773,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             H.SK[e] = (long long)((unsigned)H.r[e] * (unsigned)H.a[e] + tri32(H.r[e]));
         }
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) {
-            if (e * NWG * 32 >= n) break;  // uniform
+        for (int e = 0; e < LE; ++e) {
+            if (e * LN * 32 >= n) break;  // uniform
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const int ur = __shfl_up_sync(FULL, H.Sb[e], d), ua = __shfl_up_sync(FULL, H.kv[e], d);
@@ -779,8 +794,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         if (P.approx) dm = warp_reduce(dm, OpMin<double>());
         if (lane == 31) {  // chunk totals (chunks past the last request: zero)
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) {
-                ChSums& o = sm.ld[e * NWG + q];
+            for (int e = 0; e < LE; ++e) {
+                ChSums& o = sm.ld[e * LN + q];
                 o.A = H.kv[e];
                 o.PR = H.Sb[e];
                 o.PRA = H.SK[e];
@@ -796,10 +811,10 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         }
         group_sync();
         // chunk offsets: a scan of the E chunk totals over the lanes
-        int tA = lane < E ? sm.ld[lane].A : 0, tR = lane < E ? sm.ld[lane].PR : 0;
-        long long tX = lane < E ? sm.ld[lane].PRA : 0;
+        int tA = lane < LC ? sm.ld[lane].A : 0, tR = lane < LC ? sm.ld[lane].PR : 0;
+        long long tX = lane < LC ? sm.ld[lane].PRA : 0;
 #pragma unroll
-        for (int d = 1; d < (E < 32 ? E : 32); d <<= 1) {
+        for (int d = 1; d < LC; d <<= 1) {
             const int ur = __shfl_up_sync(FULL, tR, d), ua = __shfl_up_sync(FULL, tA, d);
             const long long ux = __shfl_up_sync(FULL, tX, d);
             if (lane >= d) {
@@ -808,12 +823,12 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 tX += ux;
             }
         }
-        const int allA = __shfl_sync(FULL, tA, E - 1);
+        const int allA = __shfl_sync(FULL, tA, LC - 1);
         own.sumP = own.sumIn = own.sumPred = own.npend = 0;
         own.wpmax = -f_inf();
         own.dmin = __longlong_as_double(0x7ff0000000000000ll);
 #pragma unroll
-        for (int k = 0; k < NWG; ++k) {
+        for (int k = 0; k < LN; ++k) {
             own.sumP += sm.ls[k][0];
             own.sumIn += sm.ls[k][1];
             own.sumPred += sm.ls[k][2];
@@ -823,13 +838,13 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         }
         H.sumP = own.sumP;
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) {
+        for (int e = 0; e < LE; ++e) {
             H.num[e] = H.sg[e] = f_inf();
-            if (e * NWG * 32 >= n) {
+            if (e * LN * 32 >= n) {
                 H.kv[e] = -CH_KV_MAX;
                 continue;
             }
-            const int ch = e * NWG + q;
+            const int ch = e * LN + q;
             // (inclusive offset of the chunk before)
             const int oR = __shfl_sync(FULL, tR, ch > 0 ? ch - 1 : 0);
             const int oA = __shfl_sync(FULL, tA, ch > 0 ? ch - 1 : 0);
@@ -850,10 +865,11 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
     };
     // (staged: from shared memory)
     auto put_staged = [&](const Hot<EPL>& H, const ChOwn& own) CH_INLINE {
+        const int q = warp % Cfg::LN;
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
-            const int x = elem(e);
-            if (e * NWG * 32 > own.n) break;  // uniform
+            const int x = (e * Cfg::LN + q) * 32 + lane;
+            if (e * Cfg::LN * 32 > own.n) break;  // uniform
             sm.str[x] = H.r[e];
             sm.sta[x] = H.a[e] | ((H.pend >> e) & 1u ? (int)0x80000000 : 0);
             sm.stS[x] = H.Sb[e];
@@ -881,7 +897,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             H.SK[e] = 0;
             H.kv[e] = -CH_KV_MAX;
             set_consts(H, e, f_inf(), 0.0f, 0.0f, 0);
-            if (e * NWG * 32 > own.n) continue;  // uniform
+            if (x >= own.n) continue;
             const int a = sm.sta[x];
             H.r[e] = sm.str[x];
             H.a[e] = a & 0x7fffffff;
@@ -1406,13 +1422,14 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 const int b = c & (CH_RING - 1);
                 rw = sm.raw[b];
                 const float4 rcv = sm.rc[b];
+                const bool staged = Cfg::staged(C.n[w]);
                 if (sm.hw[v] != NONE) leave(H);
                 ChOwn own;
-                if constexpr (Cfg::STAGE) {
-                    staged_wait<NWG>();
+                if (staged) {
+                    staged_wait<Cfg::LN + NWG>();
                     get_staged(H, own);
-                } else {
-                    load(H, own, w);
+                } else if constexpr (NWG > Cfg::LN) {
+                    load(H, own, w, IntC<NWG>());
                 }
                 const int n0 = H.n;
                 with_elems(n0 + 1, [&](auto ea) CH_INLINE { partial_sums(H, rw.y, c & 1, ea); });
@@ -1716,16 +1733,16 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             // while the hot warps write the leaving worker's table: worker w is
             // staged (or its requests fetched into L1), and the next candidates
             // are looked at among the workers other than the leaving one
-            if constexpr (Cfg::STAGE) {
-                if (warp < CH_LOOK0 + NWG) {
+            const int nw = C.n[w];
+            if (Cfg::staged(nw)) {
+                if (warp < CH_LOOK0 + Cfg::LN) {
                     Hot<EPL> H;
                     ChOwn own;
-                    load(H, own, w);
+                    load(H, own, w, IntC<Cfg::LN>());
                     put_staged(H, own);
-                    staged_arrive<NWG>();
+                    staged_arrive<Cfg::LN + NWG>();
                 }
             } else {
-                const int nw = C.n[w];
                 const long long base = (long long)w * cap;
                 for (int x = 32 * ((warp - CH_LOOK0) * 32 + lane); x < nw; x += 32 * 32 * CH_SCAN) {
                     const void* const line[] = {C.skey + base + x, C.in + base + x,
