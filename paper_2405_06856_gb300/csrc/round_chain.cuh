@@ -76,6 +76,10 @@ constexpr int CH_RING = 64;                   // candidate records in shared mem
 // and 1.68 ms, a simulation of 128 workers 25.2, 24.0 and 23.6 ms, 31 groups on 4,096
 // workers 0.96, 0.90 and 0.87 ms.
 constexpr int CH_AHEAD = 12;
+// Candidates looked at during a change of the hot worker in a simulation, where
+// most candidates change it: by the look-ahead warps that do not stage the new
+// one (elsewhere every look-ahead warp takes one).
+constexpr int CH_FIRST = 2;
 constexpr int CH_WIN = 1024;                  // rank positions kept in shared memory
 constexpr int CH_SORT_MAX = 2048;             // workers a trace-mode round ranks by itself
 constexpr int CH_MAX_SLOTS = 4096;            // modified workers held, at most
@@ -97,9 +101,9 @@ struct ChCfg {
     // look-ahead warps that load the next hot worker, their elements a lane, and
     // the requests that they hold
     static constexpr int LN = 4, LE = EPL, LCAP = 32 * LN * LE;
-    static __device__ __forceinline__ bool staged(int n)
+    static __device__ __forceinline__ bool staged(int n, bool sim)
     {
-        return NWG == LN || (n > 128 && n < LCAP);
+        return NWG == LN || (n < LCAP && (sim || n > 128));
     }
 };
 
@@ -1358,7 +1362,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
     // (one role's registers are not live in another's code): look ahead if
     // nothing is, links beside more look-ahead, and after a miss the change of
     // places.
-    int c = 0, alt_end = 0;
+    int c = 0, alt_end = 0, span = CH_SCAN;
+    const int first = sim ? CH_FIRST : CH_SCAN;
     int stop_at = n_cand;
     // at the end the hot workers' tables are brought up to date (a simulation's
     // next step rebuilds every table, unless Algorithm 2 reads them first)
@@ -1390,7 +1395,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                     partial_sums(H, sm.rec[(c + 1) & (CH_RING - 1)].ri, (c + 1) & 1, ea);
                 });
                 won = false;
-                alt_end = min(c + CH_SCAN, n_cand);
+                alt_end = min(c + first, n_cand);
+                span = sim ? CH_SCAN : CH_AHEAD;
                 votes_sync();  // the sums are in: CH_TERMS forms candidate c's terms
                 cta_sync();
             }
@@ -1405,12 +1411,13 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                              H.n + 1 <= decltype(ea)::value * 32 * NWG);
                 });
             if (d == CH_END && k < alt_end) votes_sync();  // CH_TERMS learns of it
-            const int new_end = min(alt_end + CH_AHEAD, n_cand);
+            const int new_end = min(alt_end + span, n_cand);
             cta_sync();
             const int code = sm.code[rp];
             c = sm.next[rp];
             if (code == CH_DONE) {
                 alt_end = new_end;
+                span = CH_AHEAD;
                 continue;
             }
             if (code == CH_STOP) break;
@@ -1422,7 +1429,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 const int b = c & (CH_RING - 1);
                 rw = sm.raw[b];
                 const float4 rcv = sm.rc[b];
-                const bool staged = Cfg::staged(C.n[w]);
+                const bool staged = Cfg::staged(C.n[w], sim);
                 if (sm.hw[v] != NONE) leave(H);
                 ChOwn own;
                 if (staged) {
@@ -1505,7 +1512,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             if (alt_end <= c) {
                 rerank();
                 prev = CH_NOBODY;
-                alt_end = min(c + CH_SCAN, n_cand);
+                alt_end = min(c + first, n_cand);
+                span = sim ? CH_SCAN : CH_AHEAD;
                 votes_sync();
                 cta_sync();
             }
@@ -1599,11 +1607,12 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                         for (int i = k; i < n_cand; ++i) io.placement[c0 + i * G] = -1;
                 }
             }
-            const int new_end = min(alt_end + CH_AHEAD, n_cand);
+            const int new_end = min(alt_end + span, n_cand);
             cta_sync();
             c = k;
             if (code == CH_DONE) {
                 alt_end = new_end;
+                span = CH_AHEAD;
                 continue;
             }
             if (code == CH_STOP) break;
@@ -1649,7 +1658,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         bool owed = false;  // the slot took the last run's last candidate
         for (int rp = 0; c < n_cand; rp ^= 1) {
             if (alt_end <= c) {
-                alt_end = min(c + CH_SCAN, n_cand);
+                alt_end = min(c + first, n_cand);
+                span = sim ? CH_SCAN : CH_AHEAD;
                 votes_sync();
                 terms(o, c, false, false);
                 cta_sync();
@@ -1668,13 +1678,14 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 owed = false;
                 __syncwarp();
             }
-            const int new_end = min(alt_end + CH_AHEAD, n_cand);
+            const int new_end = min(alt_end + span, n_cand);
             if (!(lane & 1) && lane >> 1 < KH) sm.own[lane >> 1] = o;
             cta_sync();
             const int code = sm.code[rp];
             c = sm.next[rp];
             if (code == CH_DONE) {
                 alt_end = new_end;
+                span = CH_AHEAD;
                 owed = sm.dec[(c - 1) & 1] == lane >> 1;
                 if (owed) take(c - 1);
                 continue;
@@ -1695,13 +1706,14 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         int written = 0;      // candidates whose outcomes are written
         for (int rp = 0; c < n_cand; rp ^= 1) {
             if (alt_end <= c) {
-                alt_end = min(c + CH_SCAN, n_cand);
-                const int k = c + warp - CH_LOOK0;
-                if (!primed && k < alt_end) look(k, &sm.never);
+                alt_end = min(c + first, n_cand);
+                span = sim ? CH_SCAN : CH_AHEAD;
+                const int k = c + warp - (CH_WARPS - first);
+                if (!primed && k >= c && k < alt_end) look(k, &sm.never);
                 primed = false;
                 cta_sync();
             }
-            const int new_end = min(alt_end + CH_AHEAD, n_cand);
+            const int new_end = min(alt_end + span, n_cand);
             const int rec_new = max(rec_end, min(n_cand, new_end + CH_AHEAD));
             if (clerk) {
                 flush(written, c);  // (their records are in the ring until fetch takes their place)
@@ -1721,6 +1733,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             c = sm.next[rp];
             if (code == CH_DONE) {
                 alt_end = new_end;
+                span = CH_AHEAD;
                 continue;
             }
             if (code == CH_STOP) break;
@@ -1734,7 +1747,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             // staged (or its requests fetched into L1), and the next candidates
             // are looked at among the workers other than the leaving one
             const int nw = C.n[w];
-            if (Cfg::staged(nw)) {
+            if (Cfg::staged(nw, sim)) {
                 if (warp < CH_LOOK0 + Cfg::LN) {
                     Hot<EPL> H;
                     ChOwn own;
@@ -1754,12 +1767,13 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 }
             }
             c += 1;
-            const int k = c + warp - CH_LOOK0;
-            if (k < n_cand) look(k, &sm.never);
+            const int k = c + warp - (CH_WARPS - first);
+            const bool mine = k >= c && k < n_cand;
+            if (mine) look(k, &sm.never);
             cta_sync();
             if (sm.hw[v] != NONE) {  // now the one that left
                 const int i = sm.hm[v], n = sm.left_n, b = k & (CH_RING - 1);
-                if (k < n_cand) {
+                if (mine) {
                     const CandRec cq = sm.rec[b];
                     const int ow = mw[i];
                     const unsigned long long ok = mkey[i];
