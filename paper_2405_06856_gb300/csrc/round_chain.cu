@@ -14,13 +14,18 @@ bool chain_serves_sim_e(int W, int cap, int K, int smem_max);
 
 constexpr size_t CH_FLAGS_MAX = (size_t)512 << 20;  // bytes of rank-order flags a chunk holds
 
-// Workers below which a direct round evaluates workers as it goes instead of
-// scoring every pair first.
-constexpr int CH_FLAGS_MIN_W = 192;
+// Whether a direct round scores every pair first (a launch, then a look is a
+// scan of one row of flags) or its look-ahead evaluates workers as it goes.
+// Calls of 64 candidates, with flags / without, us: 64 workers 140 / 139 (128
+// slots) and 175 / 195 (512), 128 workers 176 / 188 and 154 / 245, 512 workers
+// 189 / 271 and 188 / 852; of 16 candidates: 64 workers 82 / 77 and 105 / 111, 256
+// workers 116 / 125 and 99 / 162. The line lies where they meet.
+constexpr int CH_FLAGS_MIN_W = 64;
+constexpr long long CH_FLAGS_MIN_PAIRS = 4096;
 
 static bool ch_flags(const ClusterDev& C, const RoundIO& io)
 {
-    return C.W >= CH_FLAGS_MIN_W && io.n_cand >= 64;
+    return C.W >= CH_FLAGS_MIN_W && (long long)C.W * io.n_cand >= CH_FLAGS_MIN_PAIRS;
 }
 
 size_t round_chain_flag_bytes(const DevParams& P, const ClusterDev& C, const RoundIO& io)

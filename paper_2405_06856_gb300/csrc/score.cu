@@ -676,9 +676,12 @@ __global__ void __launch_bounds__(DIRECT_THREADS) k_score_direct(DirectArgs A)
         A.argbest[c] = !valid ? -2 : best == 0xffffffffu ? -1 : C.order[best];
 }
 
-// Calls that k_score_direct serves: up to about a million pairs (there both
-// ways take the same time) on fleets whose row searches a CTA finishes in a
-// few steps.
+// Calls that k_score_direct serves. Direct / sorted, us a call: 2^16 pairs on 64
+// workers 18 / 78, on 1,024 20 / 149; 2^19 on 256 workers 26 / 78, on 2,048 29 /
+// 107; 2^20 39 / 67 on 64 workers, 44 / 75 on 1,024, 43 / 88 on 2,048; 2^21 60 /
+// 73, 66 / 69 and 68 / 80. A heartbeat hides the sorted path's candidate sort
+// (about 25 us) behind the table build, so the line lies at 2^20, where the
+// direct path leads by more than that.
 constexpr long long DIRECT_PAIRS = 1ll << 20;
 constexpr int DIRECT_MAX_W = 2048;
 

@@ -155,7 +155,11 @@ static cudaError_t allow_smem(size_t smem)
 }
 
 constexpr int COOP_NW = 8;
-constexpr int FEW_WORKERS = 608;  // four CTAs an SM: every worker's build starts at once
+// Fleets built in one launch, a CTA a worker (four CTAs an SM: every build starts
+// at once). A load, this way / first level and list, us: 256 workers 22 / 25 (64
+// requests, 128 slots), 26 / 36 (200, 512) and 37 / 46 (500, 1,024); 608 workers
+// 24 / 25, 34 / 38 and 55 / 57; 1,216 workers 28 / 26, 44 / 44 and 78 / 71.
+constexpr int FEW_WORKERS = 608;
 
 template <int E>
 static cudaError_t build_e(const DevParams& P, const ClusterDev& C, const int32_t* list, int count,

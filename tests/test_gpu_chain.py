@@ -27,10 +27,10 @@ REFUSED = -2
 HIST = dict(lo_ms=8.0, hi_ms=20.0)
 
 # W, slots, requests a worker at first (at most), KV, candidates, parameters.
-# A hot worker's lanes hold one request more at every 128 (more than four a
-# lane: 512 slots and up step at 256, 384, 512), so the first rows fill
-# workers across those counts; the others are the dispatch's edges (192
-# workers, 64 candidates) and the options.
+# A hot worker's lanes hold one request more at every 128 (at every 256 on 1,024
+# slots, where 129 to 511 requests are staged), so the first rows fill
+# workers across those counts; the others are the dispatch's edges (64 workers,
+# 4,096 pairs a call) and the options.
 ROUNDS = {
     "slots32": (40, 32, 8, 9000, 300, dict(T_pre=200.0)),
     "slots128": (12, 128, 60, 50000, 500, LOOSE),
@@ -38,10 +38,10 @@ ROUNDS = {
     "slots512-over-128-256-384": (4, 512, 250, 240000, 900, LOOSE),
     "slots1024-over-256-384-512": (3, 1024, 380, 420000, 1500, LOOSE),
     "slots1024-fill": (8, 1024, 10, 60000, 900, dict(T_pre=150.0)),
-    "table-191": (191, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
-    "flags-192": (192, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
-    "table-63": (700, 128, 30, 40000, 63, dict(T_pre=300.0, T_dec=20.0)),
-    "flags-64": (700, 128, 30, 40000, 64, dict(T_pre=300.0, T_dec=20.0)),
+    "table-63-workers": (63, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
+    "flags-64-workers": (64, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
+    "table-4095-pairs": (195, 128, 30, 40000, 21, dict(T_pre=300.0, T_dec=20.0)),
+    "flags-4096-pairs": (256, 128, 30, 40000, 24, dict(T_pre=300.0, T_dec=20.0)),
     "flags-many-words": (1100, 64, 20, 20000, 600, dict(T_pre=200.0, T_dec=11.0)),
     "one-candidate": (20, 128, 30, 40000, 1, {}),
     "one-worker-fills": (1, 256, 30, 30000, 150, LOOSE),
