@@ -30,16 +30,16 @@
 // change places: the hot worker used least recently leaves, its table formed
 // from its aggregates (the same values as a table build's, without its sorts
 // and sums), while look-ahead warps load and sum the new worker's requests (its
-// sorted keys are kept by every table build; beyond 512 slots the hot warps do
-// that themselves afterwards) and look at the next candidates among the others.
+// sorted keys are kept by every table build) and look at the next candidates
+// among the others.
 //
 // Bound: the link's latency, a chain of dependent register arithmetic, a vote,
 // two barriers and a reduction at 45% of the SM's issue slots. On tables of up
-// to 128, 512 and 1,024 slots a plain link takes 1,150, 1,300 and 1,790 cycles
-// and a miss 7,000, 11,000 and 28,000. Measured against rebuilding the winner's
-// table at every link: 2,048 candidates on 256 workers 5.3 -> 1.68 ms, 13,107 on
-// 16,384 workers (1,024 slots) 84 -> 18 ms, 31 groups on 4,096 workers 2.75 ->
-// 0.87 ms, a simulation of 128 workers 37.2 -> 23.6 ms.
+// to 128 and 512 slots a plain link takes 1,150 and 1,300 cycles and a miss 7,000
+// and 11,000. Measured against rebuilding the winner's table at every link: 2,048
+// candidates on 256 workers 5.3 -> 1.68 ms, 13,107 on 16,384 workers (1,024
+// slots) 84 -> 17.5 ms, 31 groups on 4,096 workers 2.75 -> 0.88 ms, a simulation
+// of 128 workers 37.2 -> 23.9 ms.
 //
 // Where the round has a candidate x worker flag matrix (direct rounds of
 // larger fleets, scored by the scoring kernel against the round-start state in
@@ -92,14 +92,20 @@ constexpr int CH_KV_MAX = 1 << 29;            // KV usage saturates here (M < 2^
 constexpr int CH_HJ_MAX = 1 << 25;            // h and j likewise: one token would exceed M
 
 // Tables of up to 128 slots share E = 4. A hot worker's requests: EPL a lane
-// over NWG warps; KH hot workers.
+// over NWG warps; KH hot workers. (1,024 slots over four warps, eight requests a
+// lane, spilled a kilobyte of registers: a change of the hot worker took 28,000
+// cycles, a round of 13,107 candidates 17.9 ms against 17.1.)
 template <int E>
 struct ChCfg {
     static constexpr int NWG = E >= 32 ? 8 : 4;
     static constexpr int EPL = E / NWG;
     static constexpr int KH = CH_HOT / NWG;
-    // look-ahead warps that load the next hot worker, their elements a lane, and
-    // the requests that they hold
+    // Look-ahead warps that load (stage) the next hot worker, their elements a
+    // lane, and the requests that they hold. On 1,024-slot tables, whose eight hot
+    // warps load a small worker themselves in little time, they do so in direct
+    // rounds up to 128 requests (the look-ahead warps have six candidates to look
+    // at then); a simulation stages all that fit (147 workers of about 90 requests
+    // 1.29 ms a heartbeat against 1.50).
     static constexpr int LN = 4, LE = EPL, LCAP = 32 * LN * LE;
     static __device__ __forceinline__ bool staged(int n, bool sim)
     {
@@ -180,13 +186,6 @@ struct ChSmem {
     ChOwn own[Cfg::KH];              // as of the latest load
     int hw[CH_HOT], hm[CH_HOT];      // hot workers and their slots when a run ends
     int hn[CH_HOT];                  // their requests when they were loaded
-    // per hot request, by element: theta T_dec r + bank, the candidate's share
-    // of its iterations and the prompt's cost (shared_time, prompt_cost_*), and
-    // h r (saturated)
-    // (in shared memory where a lane holds more than 4)
-    static constexpr int HC = Cfg::EPL > 4 ? 32 * E : 1;
-    float hb[Cfg::KH][HC], hy[Cfg::KH][HC], hd[Cfg::KH][HC];
-    int hh[Cfg::KH][HC];
     // a leaving worker's requests: keys (r << 10 | slot) before and after
     // sorting, and the rest in sorted order
     alignas(16) unsigned nkey[32 * E + 4];
@@ -281,10 +280,10 @@ struct Hot {
     long long SK[EPL];
     float num[EPL];        // prompt bound x its cost, finishing with or before the candidate
     float sg[EPL];         // slack, finishing after it
-    // (ChSmem's hb, hy, hd, hh, where the registers allow)
-    static constexpr int RC = EPL <= 4 ? EPL : 1;
-    float hb[RC], hy[RC], hd[RC];
-    int hh[RC];
+    // theta T_dec r + bank, the candidate's share of its iterations and the
+    // prompt's cost (shared_time, prompt_cost_*), and h r (saturated)
+    float hb[EPL], hy[EPL], hd[EPL];
+    int hh[EPL];
     unsigned pend;         // bit e: placed in this round
     int n, M, sumP;
     float s, inv_s, stallk;
@@ -303,7 +302,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
 {
     using Cfg = ChCfg<E>;
     constexpr int NWG = Cfg::NWG, EPL = Cfg::EPL, KH = Cfg::KH;
-    static_assert(NWG * EPL * 32 == E * 32, "the capacity is covered");
+    static_assert(NWG * EPL == E && EPL <= 4, "the capacity is covered, in registers");
     extern __shared__ __align__(16) unsigned char smraw[];
     ChSmem<E>& sm = *reinterpret_cast<ChSmem<E>*>(smraw);
     const DevParams& P = A.P;
@@ -642,34 +641,17 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         [[maybe_unused]] constexpr int CH = 32 * NWG;
         if constexpr (EPL <= 2) {
             f(IntC<EPL>());
-        } else if constexpr (EPL == 4) {
+        } else {
             if (n <= CH) f(IntC<1>());
             else if (n <= 2 * CH) f(IntC<2>());
             else f(IntC<4>());
-        } else {
-            if (n <= 2 * CH) f(IntC<2>());
-            else if (n <= 3 * CH) f(IntC<3>());
-            else if (n <= 4 * CH) f(IntC<4>());
-            else f(IntC<EPL>());
         }
     };
-    constexpr bool REG = EPL <= 4;
-    auto get_hb = [&](const Hot<EPL>& H, int e) CH_INLINE { if constexpr (REG) return H.hb[e]; else return sm.hb[hs][elem(e)]; };
-    auto get_hy = [&](const Hot<EPL>& H, int e) CH_INLINE { if constexpr (REG) return H.hy[e]; else return sm.hy[hs][elem(e)]; };
-    auto get_hd = [&](const Hot<EPL>& H, int e) CH_INLINE { if constexpr (REG) return H.hd[e]; else return sm.hd[hs][elem(e)]; };
-    auto get_hh = [&](const Hot<EPL>& H, int e) CH_INLINE { if constexpr (REG) return H.hh[e]; else return sm.hh[hs][elem(e)]; };
     auto set_consts = [&](Hot<EPL>& H, int e, float hb, float hy, float hd, int hh) CH_INLINE {
-        if constexpr (REG) {
-            H.hb[e] = hb;
-            H.hy[e] = hy;
-            H.hd[e] = hd;
-            H.hh[e] = hh;
-        } else {
-            sm.hb[hs][elem(e)] = hb;
-            sm.hy[hs][elem(e)] = hy;
-            sm.hd[hs][elem(e)] = hd;
-            sm.hh[hs][elem(e)] = hh;
-        }
+        H.hb[e] = hb;
+        H.hy[e] = hy;
+        H.hd[e] = hd;
+        H.hh[e] = hh;
     };
     // this warp's share of the sums split at ri, to sm.ps[par]
     auto partial_sums = [&](const Hot<EPL>& H, int ri, int par, auto ea) CH_INLINE {
@@ -879,9 +861,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             sm.stS[x] = H.Sb[e];
             sm.stk[x] = H.kv[e];
             sm.stK[x] = H.SK[e];
-            sm.stb[x] = get_hb(H, e);
-            sm.sty[x] = get_hy(H, e);
-            sm.std_[x] = get_hd(H, e);
+            sm.stb[x] = H.hb[e];
+            sm.sty[x] = H.hy[e];
+            sm.std_[x] = H.hd[e];
         }
         if (q == 0 && lane == 0) sm.sto = own;
     };
@@ -927,9 +909,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
 #pragma unroll
         for (int e = 0; e < EA; ++e) {
             const bool le = H.r[e] <= ri, pe = (H.pend >> e) & 1u;
-            ok = ok & ((le ? get_hh(H, e) : 0) + H.kv[e] <= (le ? Ma : H.M));
+            ok = ok & ((le ? H.hh[e] : 0) + H.kv[e] <= (le ? Ma : H.M));
             // the quotient num / cost >= a: where num - a cost >= 0 it holds
-            const float v = fmaf(-a, get_hd(H, e), H.num[e]);
+            const float v = fmaf(-a, H.hd[e], H.num[e]);
             mv = fminf(mv, le ? v : f_inf());
             mS = fminf(mS, le | pe ? f_inf() : H.sg[e]);
             mSp = fminf(mSp, le | !pe ? f_inf() : H.sg[e]);
@@ -943,14 +925,14 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         bool maybe = ok;
 #pragma unroll
         for (int e = 0; e < EA; ++e) {
-            const float d = get_hd(H, e);
+            const float d = H.hd[e];
             maybe = maybe & (H.r[e] > ri || H.r[e] == 0 ||
                              fmaf(-a, d, H.num[e]) >= -(a * d * 2.4e-7f + 1e-30f));
         }
         if (!__all_sync(FULL, maybe)) return false;
 #pragma unroll
         for (int e = 0; e < EA; ++e)
-            if (H.r[e] > 0 && H.r[e] <= ri) ok = ok & (H.num[e] / get_hd(H, e) >= a);
+            if (H.r[e] > 0 && H.r[e] <= ri) ok = ok & (H.num[e] / H.hd[e] >= a);
         return __all_sync(FULL, ok) != 0;
     };
     // bounds of a request of aggregates Sb, SK (finishing before / after the
@@ -1002,13 +984,13 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             add_to(H.r[e], a, r, Sb[e], SK[e]);
             // (unsigned)(r[e] - 1) < r: 1 <= r[e] <= r
             kv[e] = (unsigned)(H.r[e] - 1) < (unsigned)r
-                        ? min(CH_KV_MAX, H.kv[e] + ha + get_hh(H, e))
+                        ? min(CH_KV_MAX, H.kv[e] + ha + H.hh[e])
                         : H.kv[e];
             Sb[e] = fresh ? ne.Sb : Sb[e];
             SK[e] = fresh ? ne.SK : SK[e];
             kv[e] = fresh ? ne.kv : kv[e];
-            bounds(H, fresh ? r : H.r[e], Sb[e], SK[e], fresh ? rcv.y : get_hb(H, e),
-                   fresh ? rcv.z : get_hy(H, e), fresh || ((H.pend >> e) & 1u), stallk, num[e],
+            bounds(H, fresh ? r : H.r[e], Sb[e], SK[e], fresh ? rcv.y : H.hb[e],
+                   fresh ? rcv.z : H.hy[e], fresh || ((H.pend >> e) & 1u), stallk, num[e],
                    sg[e]);
         }
         partial_sums(H, ri2, par, ea);
@@ -1023,20 +1005,13 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 H.num[e] = num[e];
                 H.sg[e] = sg[e];
                 const bool fresh = elem(e) == n0;
-                if constexpr (REG) {
-                    H.r[e] = fresh ? r : H.r[e];
-                    H.a[e] = fresh ? a : H.a[e];
-                    H.pend |= fresh ? 1u << e : 0u;
-                    H.hb[e] = fresh ? rcv.y : H.hb[e];
-                    H.hy[e] = fresh ? rcv.z : H.hy[e];
-                    H.hd[e] = fresh ? cost : H.hd[e];
-                    H.hh[e] = fresh ? hr : H.hh[e];
-                } else if (fresh) {
-                    H.r[e] = r;
-                    H.a[e] = a;
-                    H.pend |= 1u << e;
-                    set_consts(H, e, rcv.y, rcv.z, cost, hr);
-                }
+                H.r[e] = fresh ? r : H.r[e];
+                H.a[e] = fresh ? a : H.a[e];
+                H.pend |= fresh ? 1u << e : 0u;
+                H.hb[e] = fresh ? rcv.y : H.hb[e];
+                H.hy[e] = fresh ? rcv.z : H.hy[e];
+                H.hd[e] = fresh ? cost : H.hd[e];
+                H.hh[e] = fresh ? hr : H.hh[e];
             }
             H.n = n0 + 1;
             H.sumP += a;
@@ -1190,7 +1165,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 sm.ekv[p] = H.kv[e];
                 sm.eSb[p] = H.Sb[e];
                 sm.eSK[p] = H.SK[e];
-                sm.ebnd[p] = H.num[e] / get_hd(H, e);
+                sm.ebnd[p] = H.num[e] / H.hd[e];
                 sm.esg[p] = H.sg[e];
             }
         hot_group_sync<NWG>();
@@ -1450,7 +1425,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                     if (e * NWG * 32 > n0) break;  // uniform
                     add_to(H.r[e], rw.x, rw.y, H.Sb[e], H.SK[e]);
                     if ((unsigned)(H.r[e] - 1) < (unsigned)rw.y)
-                        H.kv[e] = min(CH_KV_MAX, H.kv[e] + ha + get_hh(H, e));
+                        H.kv[e] = min(CH_KV_MAX, H.kv[e] + ha + H.hh[e]);
                     if (x == n0) {
                         H.r[e] = rw.y;
                         H.a[e] = rw.x;
@@ -1461,7 +1436,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                         set_consts(H, e, rcv.y, rcv.z, prompt_cost_new(P, H.s, (float)rw.y),
                                    sat((long long)hc * rw.y));
                     }
-                    bounds(H, H.r[e], H.Sb[e], H.SK[e], get_hb(H, e), get_hy(H, e),
+                    bounds(H, H.r[e], H.Sb[e], H.SK[e], H.hb[e], H.hy[e],
                            (H.pend >> e) & 1u, stallk, H.num[e], H.sg[e]);
                 }
                 H.n = n0 + 1;
