@@ -939,7 +939,7 @@ def min_workers_1m(A, synth, stream):
 
 def run_aux(args):
     """Small runs of the auxiliary kernels, each warm-up + steps times on the
-    256-worker workload: a grouped best-fit round (k_round_grp, 7 groups), a
+    256-worker workload: a grouped best-fit round (7 groups, a chain each), a
     JSQ round (k_round_queue), the 100 ms execution step (k_advance) and
     Algorithm 2's re-balancing of a round (k_rebalance). The command the
     profiles of those kernels capture."""
