@@ -204,6 +204,7 @@ struct ChSmem {
     float tf[4][32];                 // and bounds
     int code[2], next[2];            // [run parity]
     int miss_w, miss_f, victim;
+    int miss_n;                      // the new hot worker's requests
     int left_n;                      // requests of the worker that left last
     int abort, never;                // a run has ended; always 0
     int cnt[CH_WARPS + 1];
@@ -694,8 +695,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         }
         return t;
     };
-    // load worker w's requests into the registers of LN warps
-    auto load = [&](auto& H, ChOwn& own, int w, auto ln) CH_INLINE {
+    // load worker w's n requests into the registers of LN warps
+    auto load = [&](auto& H, ChOwn& own, int w, int n, auto ln) CH_INLINE {
         constexpr int LN = decltype(ln)::value, LE = EPL, LC = LE * LN;
         constexpr bool HOT = LN == NWG && NWG > Cfg::LN;  // by the hot warps themselves
         const int q = warp % LN;
@@ -705,7 +706,6 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             else stage_group_sync<LN>();
         };
         const long long base = (long long)w * cap;
-        const int n = C.n[w];
         H.n = n;
         H.M = C.M[w];
         H.s = C.scale[w];
@@ -1336,7 +1336,11 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
     // Every role runs the same sequence of phases, each in a loop of its own
     // (one role's registers are not live in another's code): look ahead if
     // nothing is, links beside more look-ahead, and after a miss the change of
-    // places.
+    // places. cta_sync parts the phases, and what a role decides for itself in
+    // one (who stages the new worker, say) it decides from words that no role
+    // writes in it: counts come from sm.miss_n and mn, never from C.n, which is
+    // only written here. Inside the links' phase votes_sync and the decision's
+    // barrier order the double-buffered words; sm.abort alone is polled.
     int c = 0, alt_end = 0, span = CH_SCAN;
     const int first = sim ? CH_FIRST : CH_SCAN;
     int stop_at = n_cand;
@@ -1404,14 +1408,15 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 const int b = c & (CH_RING - 1);
                 rw = sm.raw[b];
                 const float4 rcv = sm.rc[b];
-                const bool staged = Cfg::staged(C.n[w], sim);
+                const int nw = sm.miss_n;
+                const bool staged = Cfg::staged(nw, sim);
                 if (sm.hw[v] != NONE) leave(H);
                 ChOwn own;
                 if (staged) {
                     staged_wait<Cfg::LN + NWG>();
                     get_staged(H, own);
                 } else if constexpr (NWG > Cfg::LN) {
-                    load(H, own, w, IntC<NWG>());
+                    load(H, own, w, nw, IntC<NWG>());
                 }
                 const int n0 = H.n;
                 with_elems(n0 + 1, [&](auto ea) CH_INLINE { partial_sums(H, rw.y, c & 1, ea); });
@@ -1565,6 +1570,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                     sm.miss_w = w;
                     sm.miss_f = f;
                     sm.victim = (int)(lru & 15u);
+                    const int i = f & CH_IDX;
+                    sm.miss_n = !(f & CH_UNMOD) ? mn[i] : i < nwin ? win[i].n : rank_ent[i].n;
                     // hot from here on (bit 31), so that the look-ahead leaves
                     // it out
                     if (!(f & CH_UNMOD)) {
@@ -1721,12 +1728,12 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             // while the hot warps write the leaving worker's table: worker w is
             // staged (or its requests fetched into L1), and the next candidates
             // are looked at among the workers other than the leaving one
-            const int nw = C.n[w];
+            const int nw = sm.miss_n;
             if (Cfg::staged(nw, sim)) {
                 if (warp < CH_LOOK0 + Cfg::LN) {
                     Hot<EPL> H;
                     ChOwn own;
-                    load(H, own, w, IntC<Cfg::LN>());
+                    load(H, own, w, nw, IntC<Cfg::LN>());
                     put_staged(H, own);
                     staged_arrive<Cfg::LN + NWG>();
                 }

@@ -120,6 +120,38 @@ def test_chain_places_like_the_oracle(A, orc, synth, name):
         assert np.array_equal(counts, oc.n)
 
 
+def kv_peak(wl, w):
+    """KV usage of worker w's requests at its highest."""
+    q = slice(wl.roff[w], wl.roff[w + 1])
+    r = np.sort(wl.req_pred[q] - wl.req_gen[q])
+    a = (wl.req_in[q] + wl.req_gen[q])[np.argsort(wl.req_pred[q] - wl.req_gen[q])]
+    left = np.arange(len(r), 0, -1)
+    return int((np.cumsum(a[::-1])[::-1] + r * left).max())
+
+
+def test_chain_counts_at_the_staging_lines(A, orc, synth):
+    """On 1,024 slots who loads a worker that becomes hot depends on how many
+    requests it holds: the look-ahead warps from 129 to 511, its own warps
+    otherwise. Every worker of a direct round becomes hot with a count at
+    those lines, and some again after they left."""
+    counts = np.array([126, 127, 128, 129, 130, 510, 511, 512, 513, 128, 511, 0], np.int64)
+    W, n = len(counts), 120
+    wl = synth.make_cluster("lines", 811, W, 520, 1, n, b_cap=1024, params=LOOSE)
+    rows = np.concatenate([np.arange(wl.roff[w], wl.roff[w] + counts[w]) for w in range(W)])
+    for k in ("req_in", "req_gen", "req_pred"):
+        setattr(wl, k, getattr(wl, k)[rows].copy())
+    wl.roff = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    wl.kv_capacity = np.array([(kv_peak(wl, w) if counts[w] else 0) + 2500 for w in range(W)], np.int64)
+    oc = oracle_cluster(orc, wl, None)
+    ref = oracle_round(oc, wl, 0, n)
+    assert set(ref[ref >= 0]) == set(range(W))  # every count becomes hot
+    with A.Cluster.from_workload(wl) as cl:
+        pl = cl.place_round(wl.cand_in, wl.cand_pred, wl.cand_wait)
+        assert cl.status() == A.OK
+        assert np.array_equal(pl, ref), np.argwhere(pl != ref)[:5]
+        assert np.array_equal(cl.state()[0], oc.n)
+
+
 @pytest.mark.parametrize("N,cap,kv,rate,extra", [
     (7, 64, 16000, 30.0, {}),
     (6, 128, 40000, 60.0, dict(gamma=0.3)),
