@@ -239,6 +239,9 @@ __device__ __forceinline__ void hot_group_sync()
     asm volatile("bar.sync 4, %0;" ::"r"(N * 32) : "memory");
 }
 
+// The warps looking ahead, among themselves.
+__device__ __forceinline__ void look_sync() { asm volatile("bar.sync 2, %0;" ::"n"(CH_SCAN * 32) : "memory"); }
+
 // The warps that stage a worker among themselves, and its handing over.
 template <int N>
 __device__ __forceinline__ void stage_group_sync()
@@ -1339,7 +1342,10 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
     // places. cta_sync parts the phases, and what a role decides for itself in
     // one (who stages the new worker, say) it decides from words that no role
     // writes in it: counts come from sm.miss_n and mn, never from C.n, which is
-    // only written here. Inside the links' phase votes_sync and the decision's
+    // only written here. Of the modified workers' entries mw, mn and modbits are
+    // the look-ahead warps' own, written in a change only; the rest of a slot is
+    // written by the hot warps whose worker leaves, while mn says that it is hot
+    // and nobody looks at it. Inside the links' phase votes_sync and the decision's
     // barrier order the double-buffered words; sm.abort alone is polled.
     int c = 0, alt_end = 0, span = CH_SCAN;
     const int first = sim ? CH_FIRST : CH_SCAN;
@@ -1465,6 +1471,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             c += 1;
             alt_end = c;
         }
+        cta_sync();  // (the other roles' last writes follow)
         if (last_tables) {
             cta_sync();  // the last links' logs and terms
             for (int k = 0; k < KH; ++k) {
@@ -1572,16 +1579,6 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                     sm.victim = (int)(lru & 15u);
                     const int i = f & CH_IDX;
                     sm.miss_n = !(f & CH_UNMOD) ? mn[i] : i < nwin ? win[i].n : rank_ent[i].n;
-                    // hot from here on (bit 31), so that the look-ahead leaves
-                    // it out
-                    if (!(f & CH_UNMOD)) {
-                        mn[f & CH_IDX] = (int)0x80000000;
-                    } else if (mcount < mmax) {
-                        const int pos = f & CH_IDX;
-                        mw[mcount] = w;
-                        mn[mcount] = (int)0x80000000;
-                        modbits[pos >> 5] |= 1u << (pos & 31);
-                    }
                     sm.lw_[b] = w;
                 } else if (code == CH_STOP) {
                     *io.status = -2;  // ALADDIN_ERR_CAPACITY
@@ -1617,6 +1614,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             c += 1;
             alt_end = c;
         }
+        cta_sync();  // the last phase's readers are done
         if (lane < KH) {
             sm.hw[lane] = hk_w;
             sm.hm[lane] = hk_m;
@@ -1681,6 +1679,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             c += 1;
             alt_end = c;
         }
+        cta_sync();  // the last phase's readers are done
         if (!(lane & 1) && lane >> 1 < KH) sm.own[lane >> 1] = o;
     } else {
         const bool clerk = warp == CH_WARPS - 1;  // fetches the records, writes the outcomes
@@ -1724,6 +1723,16 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 stop_at = c;
                 break;
             }
+            // hot from here on (bit 31), so that the look-ahead leaves it out
+            if (warp == CH_LOOK0 && lane == 0) {
+                mn[f & CH_UNMOD ? mcount : f & CH_IDX] = (int)0x80000000;
+                if (f & CH_UNMOD) {
+                    const int pos = f & CH_IDX;
+                    mw[mcount] = w;
+                    modbits[pos >> 5] |= 1u << (pos & 31);
+                }
+            }
+            look_sync();
             if (f & CH_UNMOD) mcount++;
             // while the hot warps write the leaving worker's table: worker w is
             // staged (or its requests fetched into L1), and the next candidates
@@ -1782,6 +1791,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             primed = true;
             alt_end = c;
         }
+        cta_sync();  // (likewise)
         if (clerk) flush(written, c);
     }
     if (last_tables && warp >= CH_HOT)
