@@ -122,15 +122,18 @@ int round_ctas(int W, int cap, int K, bool single_cta);
 
 // Scratch of the placement chain (grow-only, owned by the cluster).
 struct RoundChainBuffers {
-    uint8_t* flags;        // [chunk][(W + 31) & ~31] rank-order flags of the round-start
-                           // state, or nullptr (round_chain_flag_bytes is 0)
+    uint8_t* flags;        // [chunk][round_flag_row(W)] rank-order flags of the round-start
+                           // state, or nullptr (round_chain_chunk is 0)
+    int chunk;             // candidates that flags and score hold
     void* rank;            // [W] 16-byte rank entries
     int* c_stop;           // one int
     ScoreBuffers score;    // candidate preparation of the pre-scoring (chunk candidates)
 };
-// Bytes of the chain's flag buffer for a direct-mode round (0: it evaluates
-// workers as it goes and needs none).
-size_t round_chain_flag_bytes(const DevParams& P, const ClusterDev& C, const RoundIO& io);
+// Bytes of a candidate's row in the chain's flag buffer, and the candidates that
+// the buffer holds for a direct-mode round (0: it evaluates workers as it goes
+// and needs none); a longer round runs in chunks of as many.
+inline int round_flag_row(int W) { return (W + 31) & ~31; }
+int round_chain_chunk(const DevParams& P, const ClusterDev& C, const RoundIO& io);
 // K4 as a chain (round_chain.cu): direct-mode best-fit rounds, of one
 // scheduling group (the sliced round finishes any candidates left when the
 // modified workers outgrow shared memory) or of several (one CTA each), and

@@ -862,10 +862,10 @@ try {
         CK(cl->r_stop.ensure(sizeof(int)));
         rb.rank = cl->r_rank.p;
         rb.c_stop = cl->r_stop.as<int>();
-        const size_t fbytes = round_chain_flag_bytes(cl->dp, cl->dev, io);
-        if (fbytes > 0) {
-            const size_t chunk = fbytes / (size_t)((cl->W + 31) & ~31);
-            CK(cl->r_flags.ensure(fbytes));
+        rb.chunk = round_chain_chunk(cl->dp, cl->dev, io);
+        if (rb.chunk > 0) {
+            const size_t chunk = (size_t)rb.chunk;
+            CK(cl->r_flags.ensure(chunk * (size_t)round_flag_row(cl->W)));
             CK(cl->sorted.ensure(sizeof(float4) * CAND_REC_F4 * chunk));
             CK(cl->hist.ensure(sizeof(int32_t) * ((size_t)cl->hp.K + 2)));
             CK(cl->best.ensure(sizeof(unsigned int) * chunk));

@@ -28,12 +28,11 @@ static bool ch_flags(const ClusterDev& C, const RoundIO& io)
     return C.W >= CH_FLAGS_MIN_W && (long long)C.W * io.n_cand >= CH_FLAGS_MIN_PAIRS;
 }
 
-size_t round_chain_flag_bytes(const DevParams& P, const ClusterDev& C, const RoundIO& io)
+int round_chain_chunk(const DevParams& P, const ClusterDev& C, const RoundIO& io)
 {
-    if (io.sim || P.groups > 1 || !ch_flags(C, io)) return 0;
-    const size_t ldf = (size_t)((C.W + 31) & ~31);
-    const size_t chunk = std::min<size_t>((size_t)io.n_cand, std::max<size_t>(1, CH_FLAGS_MAX / ldf));
-    return chunk * ldf;
+    if (io.sim || P.groups > 1 || P.wait_test || !ch_flags(C, io)) return 0;
+    const size_t rows = std::max<size_t>(1, CH_FLAGS_MAX / (size_t)round_flag_row(C.W));
+    return (int)std::min<size_t>((size_t)io.n_cand, rows);
 }
 
 bool round_chain_serves_sim(int W, int cap, int K)

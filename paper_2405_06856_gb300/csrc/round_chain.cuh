@@ -87,7 +87,6 @@ constexpr int CH_RC_MAX = 64;                 // breakpoint samples of one in sh
 constexpr int CH_TSHIFT = 2;                  // without flags: every 4th breakpoint is sampled
 constexpr int CH_TS_MAX = 64;                 // samples of one, at most
 constexpr int CH_UB = 32;                     // prompt limits of one, by predicted length
-constexpr size_t CH_FLAGS_MAX = (size_t)512 << 20;  // bytes of rank-order flags a chunk holds
 constexpr int CH_KV_MAX = 1 << 29;            // KV usage saturates here (M < 2^24)
 constexpr int CH_HJ_MAX = 1 << 25;            // h and j likewise: one token would exceed M
 
@@ -1907,10 +1906,9 @@ cudaError_t round_chain_e(const DevParams& P, const ClusterDev& C, const RoundIO
         k_round_chain<E><<<G, CH_THREADS, smem, st>>>(A);
         return cudaGetLastError();
     }
-    const int ldf = (C.W + 31) & ~31;
+    const int ldf = round_flag_row(C.W);
     int chunk = io.n_cand;
-    if (B->flags)
-        chunk = (int)std::min<size_t>((size_t)io.n_cand, std::max<size_t>(1, CH_FLAGS_MAX / ldf));
+    if (B->flags) chunk = std::min(chunk, B->chunk);
     if (P.round_chunk > 0 && chunk > P.round_chunk) chunk = P.round_chunk;
     for (int c0 = 0; c0 < io.n_cand; c0 += chunk) {
         const int n = std::min(chunk, io.n_cand - c0);
