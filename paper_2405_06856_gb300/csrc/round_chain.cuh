@@ -1524,7 +1524,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 const unsigned votes =
                     __ballot_sync(FULL, lane < CH_HOT && sm.vote[par][lane & (CH_HOT - 1)] != 0);
                 constexpr unsigned all = (1u << NWG) - 1u;
-                const bool yes = own_ok != 0 && ((votes >> (lane * NWG)) & all) == all;
+                // (a shift by lane % KH: the other lanes' rank keeps them out)
+                const bool yes = own_ok != 0 && ((votes >> (lane % KH * NWG)) & all) == all;
                 const unsigned pick = __reduce_min_sync(FULL, yes ? rank : 0xffffffffu);
                 const bool hit = pick != 0xffffffffu;
                 // a worker that is not hot, or that has no free slot, ends the run
