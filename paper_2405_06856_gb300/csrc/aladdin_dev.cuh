@@ -183,6 +183,13 @@ __device__ __forceinline__ long long floor_div_ll(long long x, long long d)
     return q;
 }
 
+// Time over the latency scale that a candidate of a finishing request's r
+// iterations adds to them: its batch slot and its growing context.
+__device__ __forceinline__ float shared_time(const DevParams& P, float r)
+{
+    return fmaf(P.c2, r, __fmul_rn(P.k2, __fmul_rn(0.5f * r, __fadd_rn(r, 1.0f))));
+}
+
 __device__ __forceinline__ CandRec make_cand(const DevParams& P, int32_t in, int32_t pred, float w,
                                              int32_t orig)
 {
@@ -197,10 +204,9 @@ __device__ __forceinline__ CandRec make_cand(const DevParams& P, int32_t in, int
     c.inv_r = 1.0f / rf;
     // approximate mode: a + gamma * l_pred, the candidate's share of (b)
     c.Ua = P.approx ? fmaf(P.gamma, rf, a) : (-P.c2_over_k2 - 0.5f * (rf + 1.0f)) - a;
-    const float d1 = P.k2 * rf + P.k1;
+    const float d1 = fmaf(P.k2, rf, P.k1);
     c.inv_d1 = 1.0f / d1;
-    const float X = P.c2 * rf + P.k2 * (0.5f * rf * (rf + 1.0f));
-    c.nXd1 = -X * c.inv_d1;
+    c.nXd1 = -shared_time(P, rf) * c.inv_d1;
     c.inv_d2 = 1.0f / (P.k2 * rf);
     // decode instance: no TTFT test (the bound is +inf for every worker)
     c.Zc = P.decode ? f_inf() : (P.T_pre - (ok ? w : 0.0f)) * P.inv_k1;
@@ -529,14 +535,18 @@ __device__ __forceinline__ void add_carry_suffix(Set& st, typename Set::value_ty
 }
 
 // The terms of a table that the placement chain also forms request by request
-// (round_chain.cu): both call these, so that both round alike.
+// (round_chain.cuh). Both call these, and every product and sum states its
+// rounding: left to the compiler, a sum of two products is fused one way in one
+// place and the other way in the next, and a table that the chain leaves would
+// differ in last bits from the one built of the same requests (a restored
+// cluster's).
 
 // Cumulative decode time T(x) of iterations 1..x: Sb requests summed over the
 // iterations, SK context tokens (the product with s rounded by itself).
 __device__ __forceinline__ float decode_time(const DevParams& P, float s, float x, float Sb,
                                              float SK)
 {
-    return __fmul_rn(s, P.c3 * x + P.c2 * Sb + P.k2 * SK);
+    return __fmul_rn(s, fmaf(P.k2, SK, fmaf(P.c3, x, __fmul_rn(P.c2, Sb))));
 }
 
 // Slack sigma_j of a request of r remaining iterations that end at T; base =
@@ -550,10 +560,6 @@ __device__ __forceinline__ float slack_base(const DevParams& P, float r, float b
 // quotient: its slack less the candidate's share of its r iterations (u_j =
 // sigma_j - s * shared_time), and the stall too for one decoding at round
 // start (stallk = k1 P + c1), over the prompt's cost.
-__device__ __forceinline__ float shared_time(const DevParams& P, float r)
-{
-    return P.c2 * r + P.k2 * (0.5f * r * (r + 1.0f));
-}
 __device__ __forceinline__ float shared_slack(float s, float sigma, float shared)
 {
     return fmaf(-s, shared, sigma);
@@ -564,38 +570,49 @@ __device__ __forceinline__ float stalled_slack(float s, float u, float stallk)
 }
 __device__ __forceinline__ float prompt_cost_new(const DevParams& P, float s, float r)
 {
-    return s * P.k2 * r;
+    return __fmul_rn(__fmul_rn(s, P.k2), r);
 }
 __device__ __forceinline__ float prompt_cost_ongoing(const DevParams& P, float s, float r)
 {
-    return s * (P.k2 * r + P.k1);
+    return __fmul_rn(s, fmaf(P.k2, r, P.k1));
+}
+
+// Approximate mode: the theta-scaled decode time that a request has saved.
+__device__ __forceinline__ double saved_time(const DevParams& P, int gen, double tdec)
+{
+    return __dmul_rn(P.thetad, fma(P.T_decd, (double)gen, -tdec));
 }
 
 // Row fields of the requests finishing after the candidate and of its own
 // decode bound.
 __device__ __forceinline__ float row_gt(float smS, float inv_s, float stallk)
 {
-    return smS * inv_s - stallk;
+    return fmaf(smS, inv_s, -stallk);
 }
 __device__ __forceinline__ float row_b0n(const DevParams& P, float PR, float PRA)
 {
-    return -(P.c2_over_k2 * PR + PRA);
+    return -fmaf(P.c2_over_k2, PR, PRA);
 }
 __device__ __forceinline__ float row_b1(const DevParams& P, float inv_s, float nf, float A)
 {
-    return P.c3_over_k2 + P.c2_over_k2 * nf + A + 0.5f * nf - P.thTdec_over_k2 * inv_s;
+    return fmaf(-P.thTdec_over_k2, inv_s, fmaf(0.5f, nf, __fadd_rn(fmaf(P.c2_over_k2, nf, P.c3_over_k2), A)));
 }
 
 // Worker record without its rank: TTFT bounds (the candidate's Zc is +inf on
 // a decode instance, and so is its bound Zc / s - y).
+__device__ __forceinline__ float stall_terms(const DevParams& P, float sumP)
+{
+    return fmaf(P.k1, sumP, P.c1);
+}
 __device__ __forceinline__ float4 worker_record(const DevParams& P, float inv_s, float off,
                                                 float sumP, float wpmax, int npend)
 {
     float4 wr;
     wr.x = inv_s;
-    wr.y = P.decode ? 0.0f : off * inv_s * P.inv_k1 + P.c1_over_k1 + sumP;
+    wr.y = P.decode ? 0.0f : __fadd_rn(fmaf(__fmul_rn(off, inv_s), P.inv_k1, P.c1_over_k1), sumP);
     wr.z = (npend > 0 && !P.decode)
-               ? (P.T_pre - wpmax - off) * inv_s * P.inv_k1 - P.c1_over_k1 - sumP
+               ? __fadd_rn(fmaf(__fmul_rn(__fadd_rn(__fadd_rn(P.T_pre, -wpmax), -off), inv_s),
+                                P.inv_k1, -P.c1_over_k1), -sumP)
                : f_inf();
     wr.w = 0.0f;
     return wr;
@@ -611,11 +628,11 @@ __device__ __forceinline__ float2 approx_bounds(const DevParams& P, double s_d, 
     if (P.decode) {
         wa.x = f_inf();  // no prefill, no stall: (d) is vacuous
     } else {
-        const double tau0 = s_d * (P.k1d * (double)sumP + P.c1d);
-        wa.x = (float)((dmin - tau0) / (s_d * P.k1d));
+        const double stall = fma(P.k1d, (double)sumP, P.c1d);
+        wa.x = (float)(fma(-s_d, stall, dmin) / __dmul_rn(s_d, P.k1d));
     }
-    const double ld = (P.T_decd / s_d - P.c3d - P.c2d * (double)(n + 1)) / P.k2d;
-    wa.y = (float)(P.thetad * ld - ((double)sumIn + P.gammad * (double)sumPred));
+    const double ld = fma(-P.c2d, (double)(n + 1), __dadd_rn(P.T_decd / s_d, -P.c3d)) / P.k2d;
+    wa.y = (float)fma(P.thetad, ld, -fma(P.gammad, (double)sumPred, (double)sumIn));
     return wa;
 }
 
@@ -664,7 +681,7 @@ __device__ __forceinline__ RowVals make_row(const DevParams& P, float inv_s, int
     o.v1.x = row_b1(P, inv_s, nf, (float)A);
     o.v1.y = -0.5f * nf;
     o.v1.z = pmA;
-    o.v1.w = row_gt(smS, inv_s, P.k1 * (float)P_pend + P.c1);
+    o.v1.w = row_gt(smS, inv_s, stall_terms(P, (float)P_pend));
     o.ext = make_float2(pmAp, smSp * inv_s);
     o.aux.PM = PM;
     o.aux.SM = SM;
@@ -842,7 +859,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
             if (i < n) {  // reloaded: the preloaded registers stay short-lived
                 const long long slot = base + i;
                 if (!C.pend[slot])  // decode time saved so far, theta-scaled
-                    dmin = fmin(dmin, P.thetad * (P.T_decd * (double)C.gen[slot] - C.tdec[slot]));
+                    dmin = fmin(dmin, saved_time(P, C.gen[slot], C.tdec[slot]));
             }
         }
 #pragma unroll
@@ -1113,7 +1130,7 @@ __device__ unsigned build_table(const DevParams& P, const ClusterDev& C, int w,
     group_sync<NW>();
 
     // Per-request bounds and slacks.
-    const float stallk = P.k1 * (float)sumP + P.c1;
+    const float stallk = stall_terms(P, (float)sumP);
     float pmA[E], pmAp[E], smS[E], smSp[E];
     long long PMx[E], SMx[E];
 #pragma unroll

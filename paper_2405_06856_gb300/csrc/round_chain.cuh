@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                     nP += 1;
                     wp = fmaxf(wp, (float)C.wait[slot]);
                 } else if (P.approx) {
-                    dm = fmin(dm, P.thetad * (P.T_decd * (double)gen - C.tdec[slot]));
+                    dm = fmin(dm, saved_time(P, gen, C.tdec[slot]));
                 }
             }
             set_consts(H, e, hb, hy, hd, sat((long long)hc * H.r[e]));
@@ -972,7 +972,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         const int ri2 = sm.rec[(k + 2) & (CH_RING - 1)].ri;
         const int a = rw.x, r = rw.y, n0 = H.n;
         const int ha = sat((long long)hc * a) + jc;
-        const float stallk = P.k1 * (float)(H.sumP + a) + P.c1;
+        const float stallk = stall_terms(P, (float)(H.sumP + a));
         const float cost = prompt_cost_new(P, H.s, cq.r);
         const int hr = sat((long long)hc * r);
         int Sb[EA], kv[EA];
@@ -1428,7 +1428,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 hot_group_sync<NWG>();
                 const ChElem ne = new_elem(slot_sums(hs, c & 1), rw.x, rw.y);
                 const int ha = sat((long long)hc * rw.x) + jc;
-                const float stallk = P.k1 * (float)(H.sumP + rw.x) + P.c1;
+                const float stallk = stall_terms(P, (float)(H.sumP + rw.x));
 #pragma unroll
                 for (int e = 0; e < EPL; ++e) {
                     const int x = elem(e);

@@ -152,6 +152,35 @@ def test_chain_counts_at_the_staging_lines(A, orc, synth):
         assert np.array_equal(cl.state()[0], oc.n)
 
 
+@pytest.mark.parametrize("cap", [128, 512, 1024])
+@pytest.mark.parametrize("extra", [{}, dict(mode=1, theta=0.9), dict(gamma=0.3, h=2, j=3, k1=0.0011, k2=1.7e-4,
+                                                                    c2=0.047, c3=7.3)])
+def test_chain_tables_equal_built_ones(A, synth, cap, extra):
+    """The chain forms the tables of the workers it used from its own sums; a
+    restored cluster builds them from the requests. On workers of several
+    latency scales both score, place and execute alike, byte for byte."""
+    p = dict(dict(T_pre=300.0, T_dec=12.0), **extra)
+    wl = synth.make_cluster("built", 900 + cap, 96, 20, 60000, 1600, per_worker_random=True, b_cap=cap,
+                            gpus_cycle=(1, 2, 4) if cap == 128 else (1, 2, 4, 8), params=p)
+    h = synth.decode_history(wl, 8.0, 12.0, 5)
+    with A.Cluster.from_workload(wl, tdec_ms=h) as a, A.Cluster.from_workload(wl, tdec_ms=h) as b:
+        pl = a.place_round(wl.cand_in[:900], wl.cand_pred[:900], wl.cand_wait[:900])
+        used = np.unique(pl[pl >= 0])
+        assert len(used) > 8 and len(np.unique(wl.lat_scale[used])) >= 3
+        A.aladdin_cluster_restore(b.handle, A.aladdin_cluster_save(a.handle))
+        q = (wl.cand_in[900:1200], wl.cand_pred[900:1200], wl.cand_wait[900:1200])
+        sa, sb = a.score(*q), b.score(*q)
+        diff = np.argwhere(sa["margin"].view(np.int32) != sb["margin"].view(np.int32))
+        assert len(diff) == 0, (len(diff), sa["margin"][tuple(diff[0])], sb["margin"][tuple(diff[0])])
+        assert np.array_equal(sa["flags"], sb["flags"]) and np.array_equal(sa["argbest"], sb["argbest"])
+        outs = []
+        for cl in (a, b):
+            pl = cl.place_round(wl.cand_in[900:], wl.cand_pred[900:], wl.cand_wait[900:])
+            cl.advance(100.0)
+            outs.append([pl.tobytes()] + [x.tobytes() for x in cl.state()])
+        assert outs[0] == outs[1]
+
+
 @pytest.mark.parametrize("N,cap,kv,rate,extra", [
     (7, 64, 16000, 30.0, {}),
     (6, 128, 40000, 60.0, dict(gamma=0.3)),
