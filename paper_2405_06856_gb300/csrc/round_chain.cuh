@@ -80,6 +80,8 @@ constexpr int CH_AHEAD = 12;
 // most candidates change it: by the look-ahead warps that do not stage the new
 // one (elsewhere every look-ahead warp takes one).
 constexpr int CH_FIRST = 2;
+// Rows of 512 flags that a look has in flight past the first.
+constexpr int CH_ROWS = 4;
 constexpr int CH_WIN = 1024;                  // rank positions kept in shared memory
 constexpr int CH_SORT_MAX = 2048;             // workers a trace-mode round ranks by itself
 constexpr int CH_MAX_SLOTS = 4096;            // modified workers held, at most
@@ -506,26 +508,33 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         if (cq.valid) {
             const int grp = filter ? sm.raw[b].w : 0;
             if (A.F) {
+                // 512 positions first (most candidates end there), then 2,048 at a
+                // time: the row's loads are what a long scan waits for
                 const uint8_t* row = A.F + (size_t)k * A.ldf;
-                for (int base = 0; base < W; base += 512) {
-                    const int p0 = base + 16 * lane;
-                    unsigned bits = 0;
-                    if (p0 < W) {
-                        bits = base == 0 ? sm.frow[b][lane]
-                                         : feasible16(__ldg(reinterpret_cast<const uint4*>(row + p0)));
-                        bits &= ~(modbits[p0 >> 5] >> (p0 & 16)) & 0xffffu;
-                        if (W - p0 < 16) bits &= (1u << (W - p0)) - 1u;
-                    }
+                int pos = -1;
+                auto open = [&](unsigned bits, int p0) CH_INLINE {  // the first one open from p0 on
+                    if (p0 < W) bits &= ~(modbits[p0 >> 5] >> (p0 & 16)) & 0xffffu;
+                    if (W - p0 < 16) bits &= W > p0 ? (1u << (W - p0)) - 1u : 0u;
                     const unsigned who = __ballot_sync(FULL, bits != 0);
-                    if (who) {
-                        const int src = __ffs(who) - 1;
-                        const int pos = __shfl_sync(FULL, p0 + __ffs(bits) - 1, src);
-                        const RankEnt e = pos < nwin ? win[pos] : rank_ent[pos];
-                        bk = e.key;
-                        bw = e.w;
-                        bf = pos | CH_UNMOD | (e.n >= cap ? CH_FULL : 0);
-                        break;
+                    if (who) pos = __shfl_sync(FULL, p0 + __ffs(bits) - 1, __ffs(who) - 1);
+                };
+                open(sm.frow[b][lane], 16 * lane);
+                for (int base = 512; base < W && pos < 0; base += 512 * CH_ROWS) {
+                    uint4 u[CH_ROWS];
+#pragma unroll
+                    for (int j = 0; j < CH_ROWS; ++j) {
+                        const int p0 = base + 512 * j + 16 * lane;
+                        u[j] = p0 < W ? __ldg(reinterpret_cast<const uint4*>(row + p0)) : uint4{0, 0, 0, 0};
                     }
+#pragma unroll
+                    for (int j = 0; j < CH_ROWS; ++j)
+                        if (pos < 0) open(feasible16(u[j]), base + 512 * j + 16 * lane);
+                }
+                if (pos >= 0) {
+                    const RankEnt e = pos < nwin ? win[pos] : rank_ent[pos];
+                    bk = e.key;
+                    bw = e.w;
+                    bf = pos | CH_UNMOD | (e.n >= cap ? CH_FULL : 0);
                 }
             } else {
                 for (int base = 0; base < W; base += 32) {

@@ -152,6 +152,26 @@ def test_chain_counts_at_the_staging_lines(A, orc, synth):
         assert np.array_equal(cl.state()[0], oc.n)
 
 
+@pytest.mark.parametrize("W", [512, 513, 2560, 2561, 4608, 4609, 5120])
+def test_chain_finds_the_last_workers(A, orc, synth, W):
+    """Every worker but the lightest is full: the scan of a candidate's flags
+    runs to the end of the row, at the edges of its steps."""
+    n = 40
+    wl = synth.make_cluster("last", W, W, 3, 1, n, b_cap=32, params=LOOSE)
+    empty = np.array([0, W // 2, W - 1])
+    keep = np.repeat(~np.isin(np.arange(W), empty), 3)
+    for k in ("req_in", "req_gen", "req_pred"):
+        setattr(wl, k, getattr(wl, k)[keep].copy())
+    wl.roff = np.concatenate([[0], np.cumsum(np.where(np.isin(np.arange(W), empty), 0, 3))]).astype(np.int32)
+    wl.kv_capacity = np.where(np.isin(np.arange(W), empty), 6000, 10).astype(np.int64)
+    oc = oracle_cluster(orc, wl, None)
+    ref = oracle_round(oc, wl, 0, n)
+    assert set(ref) == {-1, *empty}
+    with A.Cluster.from_workload(wl) as cl:
+        pl = cl.place_round(wl.cand_in, wl.cand_pred, wl.cand_wait)
+        assert np.array_equal(pl, ref), np.argwhere(pl != ref)[:5]
+
+
 @pytest.mark.parametrize("cap", [128, 512, 1024])
 @pytest.mark.parametrize("extra", [{}, dict(mode=1, theta=0.9), dict(gamma=0.3, h=2, j=3, k1=0.0011, k2=1.7e-4,
                                                                     c2=0.047, c3=7.3)])
