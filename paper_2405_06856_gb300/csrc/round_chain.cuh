@@ -71,8 +71,8 @@ constexpr int CH_TERMS = CH_HOT + 1;          // the warp that forms the workers
 constexpr int CH_LOOK0 = CH_HOT + 2;          // first warp looking ahead
 constexpr int CH_SCAN = CH_WARPS - CH_LOOK0;  // warps looking ahead
 constexpr int CH_RING = 64;                   // candidate records in shared memory
-// Candidates looked ahead at a time: a miss makes looks useless, and looks slow
-// the links beside them. 30, 18 and 12 took a round of 256 workers 1.82, 1.67
+// Candidates looked ahead at a time: a miss ends looks that are under way, and
+// looks slow the links beside them. 30, 18 and 12 took a round of 256 workers 1.82, 1.67
 // and 1.68 ms, a simulation of 128 workers 25.2, 24.0 and 23.6 ms, 31 groups on 4,096
 // workers 0.96, 0.90 and 0.87 ms.
 constexpr int CH_AHEAD = 12;
@@ -173,6 +173,7 @@ struct ChSmem {
     unsigned short frow[CH_RING][32];  // feasible bits of rank positions 0..511
     unsigned long long alt_k[CH_RING];  // best choice among the workers not hot
     int alt_w[CH_RING], alt_f[CH_RING];
+    int alt_at[CH_RING];             // 1 + the candidate it was looked at for, or 0
     int lw_[CH_RING], ln[CH_RING];   // log: each candidate's worker (-1, -2) and slot
     // by candidate parity, double-buffered
     ChSums ps[2][CH_HOT];            // each hot warp's partial sums
@@ -461,6 +462,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
     if (A.F && warp >= CH_LOOK0)
         for (int k = warp - CH_LOOK0; k < rec_end; k += CH_SCAN) fetch_row(k);
     if (tid == 0) sm.abort = sm.never = 0;
+    if (tid < CH_RING) sm.alt_at[tid] = 0;
     __syncthreads();
 
     int mcount = 0;  // modified workers (every thread tracks the same value)
@@ -520,6 +522,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 };
                 open(sm.frow[b][lane], 16 * lane);
                 for (int base = 512; base < W && pos < 0; base += 512 * CH_ROWS) {
+                    if (stopped()) return;
                     uint4 u[CH_ROWS];
 #pragma unroll
                     for (int j = 0; j < CH_ROWS; ++j) {
@@ -587,6 +590,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             const unsigned long long uk = bk;  // the unmodified worker's, the same in every lane
             const int uw = bw;
             for (int i0 = 0; i0 < mcount; i0 += 32) {
+                if ((i0 & 127) == 96 && stopped()) return;
                 const int i = i0 + lane;
                 bool on = i < mcount && mn[i] >= 0;  // not hot
                 if (on) {
@@ -617,6 +621,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             sm.alt_k[b] = bk;
             sm.alt_w[b] = bw;
             sm.alt_f[b] = bf;
+            sm.alt_at[b] = k + 1;
         }
     };
 
@@ -1691,16 +1696,59 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         cta_sync();  // the last phase's readers are done
         if (!(lane & 1) && lane >> 1 < KH) sm.own[lane >> 1] = o;
     } else {
+        // a lane holds candidate k's look against the worker that left slot v
+        auto hold_against = [&](int k, int v, int w) CH_INLINE {
+            const int b = k & (CH_RING - 1);
+            const int i = sm.hm[v], ow = sm.hw[v], n = sm.left_n;
+            bool held = sm.alt_at[b] == k + 1;
+            if (held && sm.alt_w[b] == w) {
+                held = false;
+                sm.alt_at[b] = 0;
+            }
+            const CandRec cq = sm.rec[b];
+            if (held && ow != NONE && cq.valid && (!filter || ow % GP == sm.raw[b].w)) {
+                const unsigned long long ok = mkey[i];
+                if (sm.alt_w[b] == NONE || ok > sm.alt_k[b] ||
+                    (ok == sm.alt_k[b] && ow < sm.alt_w[b])) {
+                    const long long rb = (long long)ow * C.rows;
+                    const long long row = rb + slot_row(i, rb, mR[i], cq.ri);
+                    const float4* t = C.tab + row * ROW_F4;
+                    float m;
+                    if (eval_pair_mode(P.approx != 0, t[0], t[1], C.tab2[row], mwrec[i],
+                                       P.approx ? C.wapx[ow] : make_float2(0.0f, 0.0f), cq,
+                                       m) == 15u) {
+                        sm.alt_k[b] = ok;
+                        sm.alt_w[b] = ow;
+                        sm.alt_f[b] = i | (n >= cap ? CH_FULL : 0);
+                    }
+                }
+            }
+            if (lane == 0 && ow != NONE) mn[i] = n;  // not hot any more
+        };
         const bool clerk = warp == CH_WARPS - 1;  // fetches the records, writes the outcomes
-        bool primed = false;  // the first candidates were looked at during the last miss
-        int written = 0;      // candidates whose outcomes are written
-        for (int rp = 0; c < n_cand; rp ^= 1) {
+        int written = 0;  // candidates whose outcomes are written
+        bool change = false;  // in a change of the hot worker: slot v takes worker w
+        int v = 0, w = NONE;
+        for (int rp = 0; c < n_cand || change; rp ^= 1) {
             if (alt_end <= c) {
+                // The next candidates. Looks made before stay right unless they found
+                // the worker that is hot now (they are made again), but for the
+                // worker that leaves, whose new table they are held against once it
+                // is there. (Made afresh at every miss they cost rounds that use
+                // many workers of large fleets up to half of their time: 218
+                // candidates on 14,000 workers of 128 slots 2.0 ms, 1.44 so.)
+                const int k = c + warp - (CH_WARPS - first);
+                if (k >= c && k < n_cand &&
+                    !(sm.alt_at[k & (CH_RING - 1)] == k + 1 && sm.alt_w[k & (CH_RING - 1)] != w))
+                    look(k, &sm.never);
+                if (change) {
+                    cta_sync();
+                    if (warp == CH_LOOK0) hold_against(c + lane, v, w);
+                    change = false;
+                    if (c >= n_cand) break;
+                }
                 alt_end = min(c + first, n_cand);
                 span = sim ? CH_SCAN : CH_AHEAD;
-                const int k = c + warp - (CH_WARPS - first);
-                if (!primed && k >= c && k < alt_end) look(k, &sm.never);
-                primed = false;
                 cta_sync();
             }
             const int new_end = min(alt_end + span, n_cand);
@@ -1715,6 +1763,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 for (int k = rec_end + warp - CH_LOOK0; k < rec_new; k += CH_SCAN) fetch_row(k);
             rec_end = rec_new;
             for (int k = alt_end + warp - CH_LOOK0; k < new_end; k += CH_SCAN) {
+                if (sm.alt_at[k & (CH_RING - 1)] == k + 1) continue;
                 if (__any_sync(FULL, *(volatile int*)&sm.abort)) break;
                 look(k, &sm.abort);
             }
@@ -1727,7 +1776,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 continue;
             }
             if (code == CH_STOP) break;
-            const int f = sm.miss_f, v = sm.victim, w = sm.miss_w;
+            const int f = sm.miss_f;
+            v = sm.victim;
+            w = sm.miss_w;
             if ((f & CH_UNMOD) && mcount == mmax) {
                 stop_at = c;
                 break;
@@ -1766,38 +1817,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                         asm volatile("prefetch.global.L1 [%0];" ::"l"(line[i]));
                 }
             }
+            change = true;
             c += 1;
-            const int k = c + warp - (CH_WARPS - first);
-            const bool mine = k >= c && k < n_cand;
-            if (mine) look(k, &sm.never);
-            cta_sync();
-            if (sm.hw[v] != NONE) {  // now the one that left
-                const int i = sm.hm[v], n = sm.left_n, b = k & (CH_RING - 1);
-                if (mine) {
-                    const CandRec cq = sm.rec[b];
-                    const int ow = mw[i];
-                    const unsigned long long ok = mkey[i];
-                    if (cq.valid && (sm.alt_w[b] == NONE || ok > sm.alt_k[b] ||
-                                     (ok == sm.alt_k[b] && ow < sm.alt_w[b])) &&
-                        (!filter || ow % GP == sm.raw[b].w)) {
-                        const long long rb = (long long)ow * C.rows;
-                        const long long row = rb + slot_row(i, rb, mR[i], cq.ri);
-                        const float4* t = C.tab + row * ROW_F4;
-                        float m;
-                        const unsigned fl =
-                            eval_pair_mode(P.approx != 0, t[0], t[1], C.tab2[row], mwrec[i],
-                                           P.approx ? C.wapx[ow] : make_float2(0.0f, 0.0f), cq, m);
-                        __syncwarp();
-                        if (fl == 15u && lane == 0) {
-                            sm.alt_k[b] = ok;
-                            sm.alt_w[b] = ow;
-                            sm.alt_f[b] = i | (n >= cap ? CH_FULL : 0);
-                        }
-                    }
-                }
-                if (warp == CH_LOOK0 && lane == 0) mn[i] = n;  // not hot any more
-            }
-            primed = true;
             alt_end = c;
         }
         cta_sync();  // (likewise)

@@ -54,6 +54,8 @@ ROUNDS = {
     "approx-flags": (260, 256, 40, 90000, 300,
                      dict(mode=1, theta=0.9, T_pre=200.0, T_dec=26.0, hist=1)),
     "decode": (60, 256, 40, 90000, 300, dict(phase=1, T_dec=26.0, hist=1)),
+    "flags-misses": (2600, 32, 20, 9000, 400, dict(T_pre=200.0)),
+    "table-misses": (63, 32, 20, 9000, 64, dict(T_pre=200.0)),
 }
 
 
