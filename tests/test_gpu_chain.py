@@ -56,6 +56,7 @@ ROUNDS = {
     "decode": (60, 256, 40, 90000, 300, dict(phase=1, T_dec=26.0, hist=1)),
     "flags-misses": (2600, 32, 20, 9000, 400, dict(T_pre=200.0)),
     "table-misses": (63, 32, 20, 9000, 64, dict(T_pre=200.0)),
+    "flags-fresh-start": (1200, 32, 20, 9000, 2250, dict(T_pre=200.0)),  # over 256 workers modified
 }
 
 
