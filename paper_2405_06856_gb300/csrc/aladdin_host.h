@@ -142,8 +142,9 @@ int round_chain_chunk(const DevParams& P, const ClusterDev& C, const RoundIO& io
 // launched.
 cudaError_t launch_round_chain(const DevParams& P, const ClusterDev& C, const RoundIO& io,
                                const RoundChainBuffers* B, cudaStream_t st, bool* used);
-// Whether the chain serves trace-mode rounds of W workers of cap slots.
-bool round_chain_serves_sim(int W, int cap, int K);
+// Whether the chain serves trace-mode rounds of W workers of cap slots (beside:
+// of a simulation that runs beside others, with RoundIO::single_cta set).
+bool round_chain_serves_sim(int W, int cap, int K, bool beside);
 
 // Attributes of the current device that launches size themselves by, read
 // once per device and cached (thread-safe).

@@ -1460,7 +1460,7 @@ void run_probes(const aladdin_params& p, const aladdin_worker_cfg& cfg, const De
     // probes that no single-CTA round serves must hold the cooperative token
     std::vector<char> need(probes.size(), 0);
     for (size_t k = 0; k < probes.size(); ++k)
-        need[k] = bestfit && !round_chain_serves_sim(probes[k].n, p.b_cap, p.K) &&
+        need[k] = bestfit && !round_chain_serves_sim(probes[k].n, p.b_cap, p.K, true) &&
                   round_ctas(probes[k].n, p.b_cap, p.K, true) < 0;
     auto one = [&](size_t k) {
         SimProbe* q = &probes[k];

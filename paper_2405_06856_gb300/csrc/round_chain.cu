@@ -35,8 +35,28 @@ int round_chain_chunk(const DevParams& P, const ClusterDev& C, const RoundIO& io
     return (int)std::min<size_t>((size_t)io.n_cand, rows);
 }
 
-bool round_chain_serves_sim(int W, int cap, int K)
+// Workers up to which a simulation's rounds run as a chain: its looks evaluate 32
+// workers at a time, so past a line the sliced round is faster. Alone it spans
+// several CTAs; beside others (the probes of a search) it has one. Steady
+// traces, sliced round / chain: 32 slots 0.94 at 32 workers and 0.88 at 96; 64
+// slots 0.95 and 0.93; 128 slots 1.09 at 96, 0.99-1.07 at 192, 0.90-1.03 at 256; 256
+// slots 1.05-1.18 at 192, 0.94-1.12 at 256; 512 slots 1.01-1.26 at 448, 0.72-0.96
+// at 512; 1,024 slots 0.99-1.23 at 384, 0.72-0.94 at 448.
+static int ch_sim_line(int cap, bool beside)
 {
+    switch (lanes_per_worker(cap)) {
+    case 1: return beside ? 96 : 0;
+    case 2: return beside ? 128 : 0;
+    case 4: return beside ? 256 : 192;
+    case 8: return beside ? 320 : 224;
+    case 16: return 448;
+    default: return 384;
+    }
+}
+
+bool round_chain_serves_sim(int W, int cap, int K, bool beside)
+{
+    if (W > ch_sim_line(cap, beside)) return false;
     DevInfo d;
     if (device_info(&d) != cudaSuccess) {
         cudaGetLastError();
@@ -58,6 +78,7 @@ cudaError_t launch_round_chain(const DevParams& P, const ClusterDev& C, const Ro
 {
     *used = false;
     if (P.wait_test || (!io.sim && io.n_cand <= 0) || (!io.sim && !B)) return cudaSuccess;
+    if (io.sim && C.W > ch_sim_line(C.cap, io.single_cta != 0)) return cudaSuccess;
     switch (lanes_per_worker(C.cap)) {
     case 1:
     case 2:

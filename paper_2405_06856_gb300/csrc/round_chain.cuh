@@ -83,7 +83,7 @@ constexpr int CH_FIRST = 2;
 // Rows of 512 flags that a look has in flight past the first.
 constexpr int CH_ROWS = 4;
 constexpr int CH_WIN = 1024;                  // rank positions kept in shared memory
-constexpr int CH_SORT_MAX = 2048;             // workers a trace-mode round ranks by itself
+constexpr int CH_SORT_MAX = 512;              // workers a trace-mode round ranks by itself
 constexpr int CH_MAX_SLOTS = 4096;            // modified workers held, at most
 constexpr int CH_RC_MAX = 64;                 // breakpoint samples of one in shared memory, at most
 constexpr int CH_TSHIFT = 2;                  // without flags: every 4th breakpoint is sampled

@@ -211,7 +211,16 @@ def test_chain_tables_equal_built_ones(A, synth, cap, extra):
     (3, 1024, 300000, 160.0, dict(T_dec=80.0)),
     (9, 256, 40000, 60.0, dict(rebalance=1, theta=0.9)),
     (2047, 32, 6000, 3000.0, dict(T_dec=14.0)),
-    (2049, 32, 6000, 3000.0, dict(T_dec=14.0)),   # more workers than the chain ranks by itself
+    (2049, 32, 6000, 3000.0, dict(T_dec=14.0)),
+    # both sides of the lines past which the sliced round serves
+    (192, 128, 6000, 3000.0, dict(T_dec=14.0)),
+    (193, 128, 6000, 3000.0, dict(T_dec=14.0)),
+    (224, 256, 6000, 3000.0, dict(T_dec=14.0)),
+    (225, 256, 6000, 3000.0, dict(T_dec=14.0)),
+    (448, 512, 3000, 4000.0, dict(T_dec=14.0)),
+    (449, 512, 3000, 4000.0, dict(T_dec=14.0)),
+    (384, 1024, 3000, 4000.0, dict(T_dec=14.0)),
+    (385, 1024, 3000, 4000.0, dict(T_dec=14.0)),
 ])
 def test_chain_simulates_like_the_oracle(A, orc, synth, N, cap, kv, rate, extra):
     tr = synth.diurnal_trace(40 + N, 700, rate, rate / 4)

@@ -29,9 +29,9 @@ def A():
     return aladdin
 
 
-def simulate(A, p, cfg, n, trace):
+def simulate(A, p, cfg, n, trace, cap=B_CAP):
     out = np.zeros(A.SIMULATE_OUT)
-    A.aladdin_simulate(A.make_params(p, B_CAP), cfg, int(n), trace, 100.0, 1, 0, out)
+    A.aladdin_simulate(A.make_params(p, cap), cfg, int(n), trace, 100.0, 1, 0, out)
     return out
 
 
@@ -51,3 +51,20 @@ def test_search_boundaries_hold_in_lone_simulations(A, synth):
     again = np.zeros(len(gpus), np.int32)
     A.aladdin_min_workers(A.make_params(p, B_CAP), cfgs, trace, 100.0, 4096, again)
     assert np.array_equal(got, again)
+
+
+@pytest.mark.parametrize("cap,kv,rate", [(32, 5000, 300.0), (64, 12000, 900.0), (128, 30000, 3000.0)])
+def test_search_of_small_tables_holds_in_lone_simulations(A, synth, cap, kv, rate):
+    """Tables of 32 and 64 slots, and fleets between the two lines at 128: the
+    probes of a search place with the chain where a simulation alone places
+    with the sliced round."""
+    tr = synth.diurnal_trace(12, 3000, rate, rate / 4)
+    p = dict(synth.BASE_PARAMS)
+    cfgs = A.make_cfgs([1], [kv], [1.0])
+    trace = A.make_trace(tr.t_arr, tr.req_in, tr.req_pred)
+    got = np.zeros(1, np.int32)
+    A.aladdin_min_workers(A.make_params(p, cap), cfgs, trace, 100.0, 1024, got)
+    n = int(got[0])
+    assert n > 8, n
+    assert simulate(A, p, cfgs[0], n, trace, cap)[0] == 0
+    assert simulate(A, p, cfgs[0], n - 1, trace, cap)[0] > 0
