@@ -22,7 +22,7 @@ struct GroupSmem {
     BuildSmem<EW, NW> build;
     unsigned long long bk[GR_WARPS];
     int bw[GR_WARPS];
-    int win;
+    int win, full;  // the winner (-1: none), and whether it has no free slot
 };
 
 // (key, worker): larger key, then lower index; w < 0 is "none".
@@ -90,11 +90,14 @@ __global__ void __launch_bounds__(GR_THREADS) k_round_grp(DevParams P, ClusterDe
                 const int ow = __shfl_xor_sync(FULL, bw, d);
                 gr_better(bk, bw, ok, ow);
             }
-            if (lane == 0) sm.win = bw;
+            if (lane == 0) {
+                sm.win = bw;
+                sm.full = bw >= 0 && C.n[bw] >= C.cap;
+            }
         }
         __syncthreads();
         const int win = sm.win;
-        if (win >= 0 && C.n[win] >= C.cap) {  // no free slot: the group stops
+        if (sm.full) {  // the group stops (read by every thread before the count grows)
             if (tid == 0) {
                 *io.status = -2;  // ALADDIN_ERR_CAPACITY
                 io.placement[c] = -1;

@@ -138,3 +138,41 @@ def test_features_compose(A, orc, synth, extra):
         assert out[4] == pytest.approx(ref["max_atgt"], rel=1e-12), lab
         assert int(out[6]) == ref["repredictions"] and int(out[7]) == ref["early_finishes"], lab
         assert int(out[8]) == ref["moved"], lab
+
+
+@pytest.mark.parametrize("W", [8192, 8194])
+def test_grouped_rounds_of_large_groups(A, orc, synth, W):
+    """Two groups of 4,096 workers, the most that a placement chain holds, and of
+    4,097, which k_round_grp places: like the oracle, over two calls."""
+    wl = synth.make_cluster("large", W, W, 12, 9000, 90, per_worker_random=True, b_cap=32,
+                            params=dict(T_pre=200.0, T_dec=14.0, groups=2))
+    oc = fresh_oracle(orc, wl)
+    with A.Cluster.from_workload(wl) as cl:
+        for lo, hi in ((0, 61), (61, 90)):
+            q = wl.cand_in[lo:hi], wl.cand_pred[lo:hi], wl.cand_wait[lo:hi]
+            pl = cl.place_round(*q)
+            ref = oc.place_round(*q, crid=np.arange(lo, hi))
+            assert np.array_equal(pl, ref), np.argwhere(pl != ref)[:5]
+        assert (pl >= 0).any()
+        assert np.array_equal(cl.state()[0], oc.n)
+
+
+def test_large_group_full_worker_stops_its_group(A, synth):
+    """A full worker among 4,097 of its group: the error, the candidates placed
+    before it, -1 from it on, and the other group's round to its end."""
+    W, n = 8194, 9
+    wl = synth.make_cluster("full", 3, W, 1, 10**6, n, b_cap=32,
+                            params=dict(T_pre=1e6, T_dec=1e6, groups=2))
+    counts = np.zeros(W, np.int64)
+    counts[[4, 5]] = 30, 3
+    rows = np.concatenate([np.arange(30), 30 + np.arange(3)])
+    for k in ("req_in", "req_gen", "req_pred"):
+        setattr(wl, k, getattr(wl, k)[rows].copy())
+    wl.roff = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    pl = np.full(n, 7, np.int32)
+    with A.Cluster.from_workload(wl) as cl:
+        with pytest.raises(A.AladdinError) as e:
+            A.aladdin_place_round(cl.handle, n, wl.cand_in, wl.cand_pred, wl.cand_wait, pl)
+        assert e.value.code == A.ERR_CAPACITY
+        assert pl.tolist() == [4, 5, 4, 5, -1, 5, -1, 5, -1]
+        assert cl.state()[0][[4, 5]].tolist() == [32, 7]
