@@ -105,7 +105,8 @@ struct RoundIO {
     // simulations that run side by side with others
     int single_cta;
     // direct mode: device pointer to the first candidate still to place (the
-    // ones before it were placed by the chain), or nullptr (0)
+    // ones before it were placed by the chain; with groups one entry each, counted
+    // among the group's candidates), or nullptr (0)
     const int* c_first;
     // direct mode: some worker holds requests placed earlier in the open round
     int round_open;
@@ -126,7 +127,7 @@ struct RoundChainBuffers {
                            // state, or nullptr (round_chain_chunk is 0)
     int chunk;             // candidates that flags and score hold
     void* rank;            // [W] 16-byte rank entries
-    int* c_stop;           // one int
+    int* c_stop;           // one int a group, and one more
     ScoreBuffers score;    // candidate preparation of the pre-scoring (chunk candidates)
 };
 // Bytes of a candidate's row in the chain's flag buffer, and the candidates that

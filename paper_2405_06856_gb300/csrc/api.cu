@@ -859,7 +859,7 @@ try {
         RoundChainBuffers rb;
         std::memset(&rb, 0, sizeof(rb));
         CK(cl->r_rank.ensure(16 * (size_t)cl->W));
-        CK(cl->r_stop.ensure(sizeof(int)));
+        CK(cl->r_stop.ensure(sizeof(int) * ((size_t)std::max(1, cl->dp.groups) + 1)));
         rb.rank = cl->r_rank.p;
         rb.c_stop = cl->r_stop.as<int>();
         rb.chunk = round_chain_chunk(cl->dp, cl->dev, io);

@@ -45,8 +45,10 @@ __global__ void __launch_bounds__(GR_THREADS) k_round_grp(DevParams P, ClusterDe
     const int n = io.n_cand;
     // the group's first candidate: (rid0 + c) mod G == g
     const int c0 = (int)((((long long)g - io.rid0 % G) % G + G) % G);
+    const int first = io.c_first ? io.c_first[g] : 0;  // the ones before are placed
     bool stopped = false;
-    for (int c = c0; c < n; c += G) {
+    for (long long at = c0 + (long long)first * G; at < n; at += G) {
+        const int c = (int)at;
         if (stopped) {  // CTA-uniform
             if (tid == 0) io.placement[c] = -1;
             continue;

@@ -94,6 +94,7 @@ constexpr int CH_TS_MAX = 64;                 // samples of one, at most
 // 46.7 ms without, 28.5, 24.6 and 23.0 at 768, 384 and 192; 13,107 on 16,384 (which
 // modify 204) 16.76, and 17.04 at 192.
 constexpr int CH_FRESH = 256;
+constexpr int CH_TRIAL = 48;                  // candidates before a group's chain is compared
 constexpr int CH_UB = 32;                     // prompt limits of one, by predicted length
 constexpr int CH_KV_MAX = 1 << 29;            // KV usage saturates here (M < 2^24)
 constexpr int CH_HJ_MAX = 1 << 25;            // h and j likewise: one token would exceed M
@@ -134,7 +135,10 @@ struct ChArgs {
     const uint8_t* F;    // [n_cand][ldf] flags of the round-start state, rank order, or nullptr
     int ldf;             // row stride of F (a multiple of 32)
     RankEnt* rank_ent;   // [W] scratch of rank positions beyond the ones in shared memory
-    int* c_stop;         // out (one group, direct): first candidate left to the sliced round
+    int* c_stop;         // out (direct, of each group): first candidate left to another kernel
+    int placed_cost, other_cost;  // groups: cycles that k_round_grp takes for a candidate
+                                  // that is placed and for another (0: not compared)
+    int* votes;          // groups whose chain is the slower way
     int mmax;            // modified workers held
     int rc;              // breakpoint samples of one in shared memory
     int nub;             // prompt limits of one (CH_UB + 1, or 0: none)
@@ -211,6 +215,7 @@ struct ChSmem {
     int ti[4][32];                   // a leaving worker's chunks' totals: rows, KV peaks, context
     float tf[4][32];                 // and bounds
     int code[2], next[2];            // [run parity]
+    int slow[2];                     // the rest is left to k_round_grp [same]
     int miss_w, miss_f, victim;
     int miss_n;                      // the new hot worker's requests
     int left_n;                      // requests of the worker that left last
@@ -472,6 +477,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
     __syncthreads();
 
     int mcount = 0;  // modified workers (every thread tracks the same value)
+    int c = 0;       // the next candidate
 
     // Table row of length r (rb: the worker's rows, R breakpoints) from n
     // samples of every (1 << sh)-th one: they bound it to one stretch, searched
@@ -1366,7 +1372,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
     // written by the hot warps whose worker leaves, while mn says that it is hot
     // and nobody looks at it. Inside the links' phase votes_sync and the decision's
     // barrier order the double-buffered words; sm.abort alone is polled.
-    int c = 0, alt_end = 0, span = CH_SCAN;
+    int alt_end = 0, span = CH_SCAN;
     const int first = sim ? CH_FIRST : CH_SCAN;
     int stop_at = n_cand;
     // at the end the hot workers' tables are brought up to date (a simulation's
@@ -1422,9 +1428,10 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             if (code == CH_DONE) {
                 alt_end = new_end;
                 span = CH_AHEAD;
+                if (sm.slow[rp]) break;
                 continue;
             }
-            if (code == CH_STOP) break;
+            if (code == CH_STOP || sm.slow[rp]) break;
             // a miss at candidate c: worker w becomes hot in slot v
             const int w = sm.miss_w, f = sm.miss_f, v = sm.victim;
             if ((f & CH_UNMOD) && mcount == mmax) break;  // no room for another modified worker
@@ -1514,6 +1521,9 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             }
         };
         int prev = CH_NOBODY;  // the slot that took the last candidate
+        int took = 0;          // groups: candidates placed, and when the first was taken up
+        const long long begun = A.placed_cost > 0 ? clock64() : 0;
+        bool voted = false;    // this group's chain is the slower way
         for (int rp = 0; c < n_cand; rp ^= 1) {
             if (alt_end <= c) {
                 rerank();
@@ -1565,6 +1575,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                     if (lane == 0) sm.lw_[b] = valid ? -1 : -2;
                     continue;
                 }
+                ++took;
                 const bool me = lane == d;
                 if (me) sm.lw_[b] = hk_w;
                 if (me) sm.ln[b] = hk_n;
@@ -1592,6 +1603,16 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             if (lane == 0) {
                 sm.code[rp] = code;
                 sm.next[rp] = k;
+                int slow = 0;
+                if (A.placed_cost > 0 && k >= CH_TRIAL) {
+                    if (!voted && clock64() - begun > (long long)took * A.placed_cost +
+                                                          (long long)(k - took) * A.other_cost) {
+                        voted = true;
+                        atomicAdd(A.votes, 1);
+                    }
+                    slow = 2 * *(volatile int*)A.votes >= G;
+                }
+                sm.slow[rp] = slow;
                 if (code == CH_MISS) {
                     const int w = sm.alt_w[b], f = sm.alt_f[b];
                     sm.miss_w = w;
@@ -1612,12 +1633,14 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             if (code == CH_DONE) {
                 alt_end = new_end;
                 span = CH_AHEAD;
+                if (sm.slow[rp]) break;
                 continue;
             }
-            if (code == CH_STOP) break;
+            if (code == CH_STOP || sm.slow[rp]) break;
             const int f = sm.miss_f, v = sm.victim;
             if ((f & CH_UNMOD) && mcount == mmax) break;
             if (f & CH_UNMOD) mcount++;
+            ++took;
             if (lane == 0) sm.abort = 0;
             cta_sync();
             if (lane == v) {
@@ -1688,9 +1711,10 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
                 span = CH_AHEAD;
                 owed = sm.dec[(c - 1) & 1] == lane >> 1;
                 if (owed) take(c - 1);
+                if (sm.slow[rp]) break;
                 continue;
             }
-            if (code == CH_STOP) break;
+            if (code == CH_STOP || sm.slow[rp]) break;
             const int f = sm.miss_f, v = sm.victim;
             if ((f & CH_UNMOD) && mcount == mmax) break;
             if (f & CH_UNMOD) mcount++;
@@ -1776,6 +1800,10 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
             cta_sync();
             const int code = sm.code[rp];
             c = sm.next[rp];
+            if (code != CH_STOP && sm.slow[rp]) {
+                stop_at = c;
+                break;
+            }
             if (code == CH_DONE) {
                 alt_end = new_end;
                 span = CH_AHEAD;
@@ -1834,7 +1862,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_round_chain(ChArgs A)
         for (int k = 0; k <= KH; ++k) cta_sync();
     if (warp == CH_WARPS - 1 && lane == 0) {
         if (!sim) {
-            if (A.c_stop) *A.c_stop = stop_at;
+            if (A.c_stop) A.c_stop[g] = stop_at;
         } else {
             io.counters[0] += failed;
             io.counters[1] += placed;
@@ -1861,6 +1889,27 @@ static size_t ch_smem(int W, int nwin, int mmax, int rc, int nub, int nts = 0)
            (size_t)((nwords + 3) & ~3) * 4 +
            (size_t)mmax * (16 + 8 + 4 * 3 + 4 * (size_t)nub + 2 * (size_t)(rc + R2_RHO_PAD)) +
            (nts > 0 ? (size_t)W * 2 * (size_t)(nts + R2_RHO_PAD) : 0);
+}
+
+// Groups. A chain's looks evaluate 32 workers at a time where k_round_grp evaluates
+// 512: on groups of a few hundred workers up the load decides which is faster
+// (300 candidates a group: a half-empty fleet, whose looks end early, 600 workers
+// of 128 slots a group, 3.5 ms with k_round_grp and 0.97 as a chain; nearly full
+// ones, 700 a group 3.6 and 4.5, 3,000 of 1,024 slots 22.9 and 51). So past the line
+// up to which the chain leads every group times itself against what k_round_grp
+// takes for the same candidates, and when half of the groups have taken half as
+// long again all leave the rest to it (both place alike and leave the same tables;
+// one group alone would wait for the others' chains first). The cycles: an
+// evaluation of every 512 workers 3,900 and a fixed 4,000, and a table's rebuild
+// (measured on 256 to 700 workers).
+static void ch_group_costs(int cap, int W, int* placed, int* other)
+{
+    const int line = cap <= 32 ? 160 : cap <= 64 ? 224 : cap == 512 ? 416 : 320;
+    if (W <= line) return;
+    *other = 4000 + 3900 * ((W + 511) / 512);
+    *placed = *other + (cap <= 32 ? 5500 : cap <= 64 ? 7000 : 10500);
+    *other += *other / 2;
+    *placed += *placed / 2;
 }
 
 struct ChPlan {
@@ -1931,7 +1980,8 @@ cudaError_t round_chain_e(const DevParams& P, const ClusterDev& C, const RoundIO
     A.F = nullptr;
     A.ldf = 0;
     A.rank_ent = B ? reinterpret_cast<RankEnt*>(B->rank) : nullptr;
-    A.c_stop = all ? nullptr : B->c_stop;
+    A.c_stop = io.sim ? nullptr : B->c_stop;
+    A.placed_cost = A.other_cost = 0;
     A.mmax = pl.mmax;
     A.rc = pl.rc;
     A.nub = pl.nub;
@@ -1940,8 +1990,14 @@ cudaError_t round_chain_e(const DevParams& P, const ClusterDev& C, const RoundIO
     if ((e = allow_max_smem<k_round_chain<E>>()) != cudaSuccess) return e;
     *used = true;
     if (all) {
+        if (G > 1) ch_group_costs(C.cap, Wl, &A.placed_cost, &A.other_cost);
+        A.votes = A.placed_cost > 0 ? B->c_stop + G : nullptr;
+        if (A.votes && (e = cudaMemsetAsync(A.votes, 0, sizeof(int), st)) != cudaSuccess) return e;
         k_round_chain<E><<<G, CH_THREADS, smem, st>>>(A);
-        return cudaGetLastError();
+        if ((e = cudaGetLastError()) != cudaSuccess || A.placed_cost == 0) return e;
+        RoundIO rest = io;  // (nothing where every candidate was placed)
+        rest.c_first = B->c_stop;
+        return launch_round_groups(P, C, rest, st);
     }
     const int ldf = round_flag_row(C.W);
     int chunk = io.n_cand;

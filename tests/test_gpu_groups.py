@@ -157,6 +157,29 @@ def test_grouped_rounds_of_large_groups(A, orc, synth, W):
         assert np.array_equal(cl.state()[0], oc.n)
 
 
+@pytest.mark.parametrize("b_cap,per,kv", [(32, 18, 6500), (128, 60, 22000), (1024, 60, 22000)])
+@pytest.mark.parametrize("pg,G,n", [(1000, 3, 330), (700, 5, 505), (420, 2, 260)])
+def test_groups_that_change_kernels(A, orc, synth, b_cap, per, kv, pg, G, n):
+    """Nearly full groups past the line up to which the chain leads: the chains
+    may leave the rest of a round to k_round_grp (which candidate it happens at
+    depends on time); placements, state and scores are the oracle's. Only the KV
+    limit binds, in integers, so that no pair is near."""
+    wl = synth.make_cluster("change", 60 + b_cap + pg, pg * G, per, kv, n, per_worker_random=True,
+                            b_cap=b_cap, params=dict(T_pre=1e5, T_dec=400.0, groups=G))
+    oc = fresh_oracle(orc, wl)
+    with A.Cluster.from_workload(wl) as cl:
+        cut = n - n // 5
+        for lo, hi in ((0, cut), (cut, n)):
+            q = wl.cand_in[lo:hi], wl.cand_pred[lo:hi], wl.cand_wait[lo:hi]
+            pl = cl.place_round(*q)
+            ref = oc.place_round(*q, crid=np.arange(lo, hi))
+            assert np.array_equal(pl, ref), np.argwhere(pl != ref)[:5]
+        assert np.array_equal(cl.state()[0], oc.n)
+        q = wl.cand_in[:20], wl.cand_pred[:20], wl.cand_wait[:20]
+        s, r = cl.score(*q), oc.score(*q)
+        assert np.array_equal(s["flags"] & 1, r["flags"] & 1)
+
+
 def test_large_group_full_worker_stops_its_group(A, synth):
     """A full worker among 4,097 of its group: the error, the candidates placed
     before it, -1 from it on, and the other group's round to its end."""
