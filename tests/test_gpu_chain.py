@@ -5,7 +5,7 @@ simulations; against the oracle, through the C ABI."""
 import numpy as np
 import pytest
 
-from parity import NEAR, compare_pairs
+from parity import compare_pairs
 
 pytestmark = pytest.mark.gpu
 
@@ -40,7 +40,7 @@ ROUNDS = {
     "slots1024-fill": (8, 1024, 10, 60000, 900, dict(T_pre=150.0)),
     "table-63-workers": (63, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
     "flags-64-workers": (64, 128, 30, 40000, 200, dict(T_pre=300.0, T_dec=20.0)),
-    "table-4095-pairs": (195, 128, 30, 40000, 21, dict(T_pre=300.0, T_dec=20.0)),
+    "table-4095-pairs": (195, 128, 30, 40000, 31, dict(T_pre=300.0, T_dec=20.0)),
     "flags-4096-pairs": (256, 128, 30, 40000, 24, dict(T_pre=300.0, T_dec=20.0)),
     "flags-many-words": (1100, 64, 20, 20000, 600, dict(T_pre=200.0, T_dec=11.0)),
     "one-candidate": (20, 128, 30, 40000, 1, {}),
@@ -87,13 +87,14 @@ def oracle_round(oc, wl, lo, hi):
 @pytest.mark.parametrize("name", list(ROUNDS))
 def test_chain_places_like_the_oracle(A, orc, synth, name):
     """Two calls of one open round, and scoring against the tables that the
-    chain left. A pair whose slack is within the fp32 bar of zero may go
-    either way; the first divergence, if any, must be such a pair of the
-    candidate's group."""
+    chain left (no pair that decides a placement here is within the fp32 bar of
+    zero)."""
     wl, tdec = workload(synth, name)
-    n, G = wl.n_cand, wl.params.get("groups", 1)
+    n = wl.n_cand
     oc = oracle_cluster(orc, wl, tdec)
     cut = n - n // 3
+    if name.endswith("-pairs"):  # the first call's pairs, at the edge of the dispatch
+        assert wl.n_workers * cut == int(name.split("-")[1])
     with A.Cluster.from_workload(wl, tdec_ms=tdec) as cl:
         pl, rl = [], []
         for lo, hi in ((0, cut), (cut, n)):
@@ -105,14 +106,7 @@ def test_chain_places_like_the_oracle(A, orc, synth, name):
         assert cl.status() == A.OK
         pl, rl = np.concatenate(pl), np.concatenate(rl)
         mis = np.flatnonzero(pl != rl)
-        if len(mis):
-            c = int(mis[0])
-            o2 = oracle_cluster(orc, wl, tdec)
-            oracle_round(o2, wl, 0, c)
-            r = o2.score(wl.cand_in[c:c + 1], wl.cand_pred[c:c + 1], wl.cand_wait[c:c + 1])
-            ws = np.arange(wl.n_workers)
-            assert (r["near"][0, ws % G == c % G] <= NEAR).any(), (c, pl[c], rl[c])
-            return
+        assert len(mis) == 0, (mis[0], pl[mis[0]], rl[mis[0]])
         assert (pl >= 0).any()
         k = min(n, 40)
         ok = wl.cand_pred[:k] > 0

@@ -58,8 +58,7 @@ def test_round_tiny(A, orc, synth, seed, tdec):
 
 @pytest.mark.parametrize("b_cap,seed", [(32, 205), (64, 206)])
 def test_round_small_tables(A, orc, synth, b_cap, seed):
-    """Rounds on tables of 32 and 64 slots (one and two rebuild warps, each
-    with its look-ahead group): placements and the final state equal the
+    """Rounds on tables of 32 and 64 slots: placements and the final state equal the
     oracle's, with runs of candidates on the same worker."""
     wl = synth.make_cluster("small", seed, 300, 6, 30000, 700, per_worker_random=True,
                             b_cap=b_cap, params=dict(T_pre=400.0, T_dec=10.2))
@@ -88,10 +87,10 @@ def test_round_w256(A, orc, synth):
 
 @pytest.mark.parametrize("max_slots,chunk", [(3, 0), (0, 97), (5, 131)])
 def test_round_incremental_hand_offs(A, orc, synth, max_slots, chunk):
-    """The incremental round's two hand-offs on a small cluster: with few
+    """The placement chain's two hand-offs on a small cluster: with few
     modified-worker slots the sliced round continues from the candidate that
     needs one more, and with small chunks every chunk of candidates is a
-    fresh incremental round from the current state. Both place like the
+    fresh chain from the current state. Both place like the
     oracle, over two calls (the second within the open round)."""
     wl = synth.config("w256", n_cand=900, b_cap=128)
     oc = orc.Cluster.from_workload(wl)
