@@ -355,8 +355,9 @@ int aladdin_cluster_test_waits(aladdin_cluster* cl, int64_t grid_polls, int64_t 
  * round evaluates every candidate against the round-start state and
  * re-evaluates only the workers it modifies, holding them in a bounded number
  * of shared-memory slots; when they run out, the round continues with the
- * sliced round from the current state, and very large rounds are split into
- * chunks of candidates, each a fresh chain. max_slots > 0 caps the slots and chunk > 0 the candidates per chunk,
+ * sliced round from the current state, and very large rounds, or ones that
+ * modify many workers, are split into chunks of candidates, each a fresh
+ * chain. max_slots > 0 caps the slots and chunk > 0 the candidates per chunk,
  * so that tests reach both paths on small clusters (0: the defaults). The
  * placements do not depend on either. ALADDIN_ERR_ARG for negative values. */
 int aladdin_cluster_test_round(aladdin_cluster* cl, int32_t max_slots, int32_t chunk);

@@ -137,8 +137,10 @@ inline int round_flag_row(int W) { return (W + 31) & ~31; }
 int round_chain_chunk(const DevParams& P, const ClusterDev& C, const RoundIO& io);
 // K4 as a chain (round_chain.cu): direct-mode best-fit rounds, of one
 // scheduling group (the sliced round finishes any candidates left when the
-// modified workers outgrow shared memory) or of several (one CTA each), and
-// trace-mode rounds (B unused). *used = false: not applicable (the wait test
+// modified workers outgrow shared memory) or of several (one CTA each; the
+// chains of large, nearly full groups leave candidates to launch_round_groups's
+// kernel), and trace-mode rounds (B unused). A direct round with flags that
+// modifies many workers synchronises st between its parts. *used = false: not applicable (the wait test
 // hook, or a group or simulation of more workers than one CTA holds), nothing
 // launched.
 cudaError_t launch_round_chain(const DevParams& P, const ClusterDev& C, const RoundIO& io,

@@ -8,6 +8,9 @@
 // thread evaluates a strided share of the group's workers from their table
 // rows, a block reduction picks the winner, and the build warps append the
 // request and rebuild that worker's table before the group's next candidate.
+// The placement chain (round_chain.cuh) takes such a round first; this kernel
+// serves groups of more workers than a chain holds (4,096, or what shared memory
+// takes) and what the chains of nearly full groups leave to it.
 // A group whose chosen worker has no free slot stops there (status -2); the
 // other groups go on.
 #include "aladdin_host.h"

@@ -28,8 +28,8 @@
 // modified, in the round-start capacity_norm order, and the feasible modified
 // worker of largest key). Only when that record wins (a "miss") does a worker
 // change places: the hot worker used least recently leaves, its table formed
-// from its aggregates (the same values as a table build's, without its sorts
-// and sums), while look-ahead warps load and sum the new worker's requests (its
+// from its aggregates (the bits that a table build forms, without its sorts and
+// sums), while look-ahead warps load and sum the new worker's requests (its
 // sorted keys are kept by every table build) and look at the next candidates
 // among the others.
 //
@@ -37,9 +37,12 @@
 // two barriers and a reduction at 45% of the SM's issue slots. On tables of up
 // to 128 and 512 slots a plain link takes 1,150 and 1,300 cycles and a miss 7,000
 // and 11,000. Measured against rebuilding the winner's table at every link: 2,048
-// candidates on 256 workers 5.3 -> 1.68 ms, 13,107 on 16,384 workers (1,024
-// slots) 84 -> 17.5 ms, 31 groups on 4,096 workers 2.75 -> 0.88 ms, a simulation
-// of 128 workers 37.2 -> 23.9 ms.
+// candidates on 256 workers 5.3 -> 1.70 ms, 13,107 on 16,384 workers (1,024
+// slots) 84 -> 17 ms, 31 groups on 4,096 workers 2.75 -> 0.87 ms, a simulation
+// of 128 workers 37.2 -> 23.4 ms. A round whose candidates spread over ever other
+// workers is all misses: on tables of 32 slots it is 0.7 to 0.9 times as fast as
+// rebuilding them (875 candidates on 14,000 workers 4.9 -> 6.1 ms), on larger ones
+// 0.85 to 1.3.
 //
 // Where the round has a candidate x worker flag matrix (direct rounds of
 // larger fleets, scored by the scoring kernel against the round-start state in

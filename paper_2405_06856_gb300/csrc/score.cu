@@ -781,7 +781,8 @@ static cudaError_t dispatch_vec(bool vec, bool approx, bool sf, bool smg, bool a
 }
 
 // prepare_score_kernels: every k_score instantiation dispatch_vec can reach
-// (seven output combinations x pending x tile kind x approximate) and the candidate preparation, finalize and detail kernels.
+// (seven output combinations x pending x tile kind x approximate), the
+// one-launch scoring and the candidate preparation, finalize and detail kernels.
 template <bool PEND, int TILE, bool APPROX>
 static cudaError_t prepare_vec3()
 {
