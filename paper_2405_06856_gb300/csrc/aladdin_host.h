@@ -140,9 +140,9 @@ int round_chain_chunk(const DevParams& P, const ClusterDev& C, const RoundIO& io
 // modified workers outgrow shared memory) or of several (one CTA each; the
 // chains of large, nearly full groups leave candidates to launch_round_groups's
 // kernel), and trace-mode rounds (B unused). A direct round with flags that
-// modifies many workers synchronises st between its parts. *used = false: not applicable (the wait test
-// hook, or a group or simulation of more workers than one CTA holds), nothing
-// launched.
+// modifies many workers synchronises st between its parts. *used = false: not
+// applicable (the wait test hook, a group of more workers than one CTA holds, or
+// a simulation of more than round_chain_serves_sim takes), nothing launched.
 cudaError_t launch_round_chain(const DevParams& P, const ClusterDev& C, const RoundIO& io,
                                const RoundChainBuffers* B, cudaStream_t st, bool* used);
 // Whether the chain serves trace-mode rounds of W workers of cap slots (beside:

@@ -256,7 +256,10 @@ __device__ __forceinline__ void hot_group_sync()
 }
 
 // The warps looking ahead, among themselves.
-__device__ __forceinline__ void look_sync() { asm volatile("bar.sync 2, %0;" ::"n"(CH_SCAN * 32) : "memory"); }
+__device__ __forceinline__ void look_sync()
+{
+    asm volatile("bar.sync 2, %0;" ::"n"(CH_SCAN * 32) : "memory");
+}
 
 // The warps that stage a worker among themselves, and its handing over.
 template <int N>
@@ -2029,9 +2032,8 @@ cudaError_t round_chain_e(const DevParams& P, const ClusterDev& C, const RoundIO
         k_round_chain<E><<<1, CH_THREADS, smem, st>>>(A);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (fresh) {
-            if ((e = cudaMemcpyAsync(&placed, B->c_stop, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-                (e = cudaStreamSynchronize(st)) != cudaSuccess)
-                return e;
+            e = cudaMemcpyAsync(&placed, B->c_stop, sizeof(int), cudaMemcpyDeviceToHost, st);
+            if (e != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
             if (placed <= 0) return cudaErrorUnknown;  // (a chain places CH_FRESH at least)
         } else if (pl.mmax < C.W) {
             // the sliced round places what the chain left (nothing when every
