@@ -41,7 +41,7 @@
 // slots) 84 -> 17 ms, 31 groups on 4,096 workers 2.75 -> 0.87 ms, a simulation
 // of 128 workers 37.2 -> 23.4 ms. A round whose candidates spread over ever other
 // workers is all misses: on tables of 32 slots it is 0.7 to 0.9 times as fast as
-// rebuilding them (875 candidates on 14,000 workers 4.9 -> 6.1 ms), on larger ones
+// rebuilding them (875 candidates on 14,000 workers 4.8 -> 5.9 ms), on larger ones
 // 0.85 to 1.3.
 //
 // Where the round has a candidate x worker flag matrix (direct rounds of
