@@ -140,11 +140,12 @@ def test_features_compose(A, orc, synth, extra):
         assert int(out[8]) == ref["moved"], lab
 
 
-@pytest.mark.parametrize("W", [8192, 8194])
-def test_grouped_rounds_of_large_groups(A, orc, synth, W):
-    """Two groups of 4,096 workers, the most that a placement chain holds, and of
-    4,097, which k_round_grp places: like the oracle, over two calls."""
-    wl = synth.make_cluster("large", W, W, 12, 9000, 90, per_worker_random=True, b_cap=32,
+@pytest.mark.parametrize("W,b_cap", [(8192, 32), (8194, 32), (6800, 1024), (8192, 1024)])
+def test_grouped_rounds_of_large_groups(A, orc, synth, W, b_cap):
+    """Two groups of 4,096 workers, the most that a placement chain holds (3,400
+    on 1,024 slots are held without samples or limits), and of more, which
+    k_round_grp places: like the oracle, over two calls."""
+    wl = synth.make_cluster("large", W, W, 12, 9000, 90, per_worker_random=True, b_cap=b_cap,
                             params=dict(T_pre=200.0, T_dec=14.0, groups=2))
     oc = fresh_oracle(orc, wl)
     with A.Cluster.from_workload(wl) as cl:
